@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int splits = p.k_splits > 1 ? p.k_splits : 1;
     const int kblocks = p.K / kBK / splits;          // K blocks per tile
     if (threadIdx.x == 0) {
@@ -353,20 +353,18 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        // Lane 0 waits for free stages and loads the A and B tiles.
-        int stage = 0;
-        uint32_t phase = 0;
-        bool ok = true;
-        long long issued = 0;
-        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-            const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
-            for (int kb = 0; kb < kblocks; ++kb) {
-                int go = 1;
-                if (lane == 0) go = mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag);
-                if (!__shfl_sync(0xffffffffu, go, 0)) { ok = false; break; }
-                unsigned char* sa = smem + stage * C::STAGE_BYTES;
-                unsigned char* sb = sa + C::A_BYTES;
-                if (lane == 0) {
+        // One thread waits for free stages and loads the A and B tiles.
+        if (elect_one()) {
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            long long issued = 0;
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    if (!mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
+                    unsigned char* sa = smem + stage * C::STAGE_BYTES;
+                    unsigned char* sb = sa + C::A_BYTES;
                     // the gather threads' copies complete on this barrier by their own arrivals
                     mbar_expect_tx(&full[stage], C::GATHER ? C::B_BYTES : C::STAGE_BYTES);
                     const int kx = (t.kb0 + kb) * kBK;
@@ -388,22 +386,22 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
                             tma_load_2d(sb, &p.tm_w, &full[stage], kx, t.wrow0);
                         }
                     }
+                    ++issued;
+                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
-                ++issued;
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
-        }
-        if (!ok && lane == 0) {
-            *abort_flag = 1;
-            // our own copies must land before the block exits: wait (bounded)
-            // on the full barrier of each of the last STAGES fills
-            for (long long f = issued - 1; f >= 0 && f >= issued - STAGES; --f) {
-                if (!mbar_wait(&full[f % STAGES], (uint32_t)((f / STAGES) & 1), p.err)) break;
+            if (!ok) {
+                *abort_flag = 1;
+                // our own copies must land before the block exits: wait (bounded)
+                // on the full barrier of each of the last STAGES fills
+                for (long long f = issued - 1; f >= 0 && f >= issued - STAGES; --f) {
+                    if (!mbar_wait(&full[f % STAGES], (uint32_t)((f / STAGES) & 1), p.err)) break;
+                }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(C::BM, C::BN);
             int stage = 0;
             uint32_t phase = 0;
@@ -709,7 +707,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_empty + kDecRing);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* ring = abort_flag + 1;        // [kDecRing] tile indices, -1 = no more
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tm_act)) : "memory");
         for (int s = 0; s < kDecStages; ++s) {
@@ -744,7 +742,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
 
     if (warp == 0) {
         // ------------------------------------------------ producer
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -805,7 +803,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(128, 16);
             int stage = 0;
             uint32_t phase = 0;
@@ -988,7 +986,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_consta
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     const int unit = (int)(blockIdx.x >> 1), n_units = (int)(gridDim.x >> 1);
@@ -1022,7 +1020,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_consta
 
     if (warp == 0) {
         // ------------------------------------------------ producer (both CTAs)
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -1050,7 +1048,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_consta
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (leader only)
-        if (leader && lane == 0) {
+        if (leader && elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(256, 256);
             int stage = 0;
             uint32_t phase = 0;

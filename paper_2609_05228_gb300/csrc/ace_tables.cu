@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
     uint64_t* acc_empty = acc_full + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kTabStages; ++s) {
             mbar_init(&full[s], 1);
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
     const int n_items = p.n_e * 2 * ti_n * tj_n;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(128, 256);
             int stage = 0;
             uint32_t phase = 0;
