@@ -46,9 +46,9 @@ struct TcParams {
     CUtensorMap tm_w;                   // weight rows [N * w_rows, K] bf16
     const int32_t* offsets;             // [N+1]
     const int32_t* dlist;               // [N]
-    const int4* tt_tab;                 // token tiles (expert, first row, rows, 0)
+    const int4* tt_tab;                 // token tiles (expert, first row, rows, only tile of its expert)
     const int32_t* meta;
-    void* out;                          // act bf16 [rows, m], y [rows, d] (fp32 SWAP / bf16) or logits
+    void* out;                          // act bf16 [rows, m], y [rows, d] (bf16) or logits
     int K;                              // reduction length
     int w_rows;                         // weight rows per expert (2m or d)
     int w_tiles;                        // w_rows / weight tile
@@ -68,6 +68,7 @@ struct TcParams {
     const float* ghat;                  // [T*k] g_hat by slot (GEMM 2 reads ghat[perm[r]])
     int k;
     const __nv_bfloat16* h_src;         // GEMM 1 of a prefill batch: h [T, K], rows gathered by the kernel
+    int* tile_next;                     // GEMMs on one CTA per tile: the next tile to take (zeroed by the routing)
 };
 
 // ---------------------------------------------------------------- CTA-pair (cta_group::2) helpers
@@ -140,6 +141,7 @@ struct Tile {
     int wt;       // weight tile index within the expert
     int split;    // K slice (split-K router only, else 0)
     int kb0;      // first K block of the slice
+    int once;     // non-zero: the expert's only token tile, so its weights are read once
 };
 
 // Tiles run K slice major: tile = split * n_base + (token tile * w_tiles + weight tile).
@@ -154,11 +156,13 @@ __device__ __forceinline__ Tile tile_at(const TcParams& p, int tile, int n_base,
         t.e = 0;
         t.row0 = tt * TOKTILE;
         t.nrows = min(TOKTILE, p.single_rows - t.row0);
+        t.once = 0;
     } else {
         const int4 v = p.tt_tab[tt];
         t.e = v.x;
         t.row0 = v.y;
         t.nrows = v.z;
+        t.once = v.w;
     }
     t.wrow0 = t.e * p.w_rows + wt * WTILE;
     t.wt = wt;
@@ -263,31 +267,93 @@ __device__ __forceinline__ float wide_row_ghat(const TcParams& p, const Tile& t,
     return p.ghat[p.perm[t.row0 + row]];
 }
 
+// ---------------------------------------------------------------- tile hand-out
+//
+// The grouped GEMMs are persistent: a CTA's producer thread draws tile indices
+// from a counter in global memory (zeroed by the routing), so CTAs that drew
+// light tiles draw more, and hands each index to the CTA's other roles through
+// a ring in shared memory (-1 = no more tiles).
+constexpr int kTileRing = 8;
+
+struct TileRing {
+    uint64_t* full;           // [kTileRing], one arrival (the producer)
+    uint64_t* empty;          // [kTileRing], one arrival per taker
+    volatile int* tile;       // [kTileRing]
+    int* err;
+    volatile int* abort_flag;
+};
+
+struct RingCursor {
+    int i = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next() {
+        if (++i == kTileRing) { i = 0; phase ^= 1u; }
+    }
+};
+
+__device__ __forceinline__ void ring_init(const TileRing& r, int takers) {
+    for (int i = 0; i < kTileRing; ++i) {
+        mbar_init(&r.full[i], 1);
+        mbar_init(&r.empty[i], takers);
+    }
+}
+
+// Producer: publish a tile index (or -1). False when the wait ran out.
+__device__ __forceinline__ bool ring_put(const TileRing& r, RingCursor& c, int tile) {
+    if (!mbar_wait_or_abort(&r.empty[c.i], c.phase ^ 1u, r.err, r.abort_flag)) return false;
+    r.tile[c.i] = tile;
+    mbar_arrive(&r.full[c.i]);
+    c.next();
+    return true;
+}
+
+// One thread takes the next index: >= 0, -1 (no more) or -2 (the wait ran out).
+__device__ __forceinline__ int ring_take(const TileRing& r, RingCursor& c) {
+    if (!mbar_wait_or_abort(&r.full[c.i], c.phase, r.err, r.abort_flag)) return -2;
+    const int tile = r.tile[c.i];
+    mbar_arrive(&r.empty[c.i]);
+    c.next();
+    return tile;
+}
+
+// The same for a warp (lane 0 takes).
+__device__ __forceinline__ int ring_take_warp(const TileRing& r, RingCursor& c, int lane) {
+    int tile = -2;
+    if (lane == 0) tile = ring_take(r, c);
+    else c.next();
+    return __shfl_sync(0xffffffffu, tile, 0);
+}
+
 // ---------------------------------------------------------------- kernel
 
-// SWAP: A (M = 128) = weight rows, B (N = TOKTILE) = token rows.
-// !SWAP: A (M = 128) = token rows, B (N = WTILE) = weight rows.
+// A (M = 128) = token rows, B (N = 256) = weight rows.
 // EPI 0: SwiGLU into act (bf16); EPI 1: g_hat-scaled down-projection rows
-// per slot, into y (fp32 for SWAP, bf16 otherwise); EPI 2: router logits
-// (fp32, + bias, / temperature), SWAP only.
-template <bool SWAP, int EPI, int STAGES>
+// per slot, bf16; EPI 2: router logits (fp32, + bias, / temperature).
+// EPI 0 and 1 draw their tiles from p.tile_next, in the order of the tile
+// table (fill_tile_table_mixed: tiles that read an expert's weights from HBM
+// alternate with tiles that find them in L2); EPI 2 (equal tiles) takes them
+// round-robin. Bound by the bytes in flight: an MMA thread waits about 700 of
+// 920 cycles a stage for data, as long for tiles that hit L2 as for tiles that
+// stream HBM. Drawn and interleaved tiles with the L2 hints took the gate/up
+// and down GEMMs of 8192 Zipf-routed tokens on the large layer from 2.40 to
+// 2.28 ms and 4096 tokens on the d = 2048 layer from 256 to 246 us.
+template <int EPI, int STAGES>
 struct TcCfg {
-    static constexpr int TOKTILE = SWAP ? 16 : 128;
-    static constexpr int WTILE = SWAP ? 128 : 256;
-    static constexpr int BM = 128;
-    static constexpr int BN = SWAP ? TOKTILE : WTILE;
-    static constexpr int A_ROWS = BM;
-    static constexpr int B_ROWS = BN;
-    static constexpr int A_BYTES = A_ROWS * kBK * 2;
-    static constexpr int B_BYTES = B_ROWS * kBK * 2;
+    static constexpr int TOKTILE = 128;
+    static constexpr int WTILE = 256;
+    static constexpr int A_BYTES = TOKTILE * kBK * 2;
+    static constexpr int B_BYTES = WTILE * kBK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int ACC_COLS = BN;                       // fp32 columns per accumulator
-    static constexpr int TMEM_COLS = (2 * ACC_COLS) < 32 ? 32 : 2 * ACC_COLS;
-    static constexpr int STG_BYTES = (!SWAP && EPI == 1) ? 4 * 4096 : 0;   // EPI 1 staging, 4 KB per warp
-    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/ + STG_BYTES;
+    static constexpr int ACC_COLS = WTILE;                    // fp32 columns per accumulator
+    static constexpr int TMEM_COLS = 2 * ACC_COLS;
+    static constexpr int STG_BYTES = EPI == 1 ? 4 * 4096 : 0;   // EPI 1 staging, 4 KB per warp
+    static constexpr int BAR_BYTES = 512;                     // barriers, tile ring
+    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /*align*/ + BAR_BYTES + STG_BYTES;
     // GEMM 1 of a prefill batch gathers its token rows itself: four more
     // warps copy them from h with 16-byte cp.async (no h_perm round trip)
-    static constexpr bool GATHER = !SWAP && EPI == 0;
+    static constexpr bool GATHER = EPI == 0;
+    static constexpr bool DRAW = EPI != 2;                    // tiles drawn from a counter
+    static constexpr int TAKERS = 1 + 4 + (GATHER ? 4 : 0);   // the MMA thread, the epilogue and the gather warps
     static constexpr int THREADS = GATHER ? kThreads + 32 * 4 : kThreads;
 };
 constexpr int kGatherWarp0 = kThreads / 32;      // first token-gather warp (warps 6..9)
@@ -304,17 +370,19 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <bool SWAP, int EPI, int STAGES>
-__global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert_tc(const __grid_constant__ TcParams p) {
-    using C = TcCfg<SWAP, EPI, STAGES>;
+template <int EPI, int STAGES>
+__global__ void __launch_bounds__(TcCfg<EPI, STAGES>::THREADS, 1) k_expert_tc(const __grid_constant__ TcParams p) {
+    using C = TcCfg<EPI, STAGES>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE_BYTES);
     uint64_t* empty = full + STAGES;
     uint64_t* acc_full = empty + STAGES;
     uint64_t* acc_empty = acc_full + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+    uint64_t* ring_bars = acc_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_bars + 2 * kTileRing);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const TileRing ring{ring_bars, ring_bars + kTileRing, abort_flag + 1, p.err, abort_flag};
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int splits = p.k_splits > 1 ? p.k_splits : 1;
@@ -333,6 +401,7 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
             mbar_init(&acc_full[a], 1);
             mbar_init(&acc_empty[a], 4);          // one arrival per epilogue warp
         }
+        if (C::DRAW) ring_init(ring, C::TAKERS);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -350,17 +419,40 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
     const int n_base = (p.single_rows > 0 ? (p.single_rows + C::TOKTILE - 1) / C::TOKTILE : p.meta[kMetaTokTiles]) *
                        p.w_tiles;
     const int n_tiles = n_base * splits;
+    // round-robin schedule (EPI 2): the tile after `tile`, -1 past the end
+    const auto rr_next = [&](int tile) {
+        tile = tile < 0 ? (int)blockIdx.x : tile + (int)gridDim.x;
+        return tile < n_tiles ? tile : -1;
+    };
 
     if (warp == 0) {
-        // ------------------------------------------------ TMA producer
-        // One thread waits for free stages and loads the A and B tiles.
+        // ------------------------------------------------ producer
+        // One thread draws the tiles, waits for free stages and loads the operands.
         if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
             long long issued = 0;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            RingCursor rc;
+            int tile = -1;
+            const uint64_t once_policy = l2_policy_evict_first(), reuse_policy = l2_policy_evict_normal();
+            while (true) {
+                if (C::DRAW) {
+                    // drawn once the previous tile's stages are out: its latency hides behind them
+                    tile = atomicAdd(p.tile_next, 1);
+                    if (tile >= n_tiles) tile = -1;
+                    if (!ring_put(ring, rc, tile)) { ok = false; break; }
+                } else {
+                    tile = rr_next(tile);
+                }
+                if (tile < 0) break;
                 const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
+                // the tile's two rows of 16 KB weight blocks, one block of each per stage
+                const uint8_t* w0 =
+                    p.w_tiles_hbm + (((size_t)t.e * (p.w_rows / 128) + 2 * t.wt) * p.w_kb + t.kb0) * 16384;
+                const size_t w_next = (size_t)p.w_kb * 16384;
+                // weights that one tile reads give way in L2 to those that more tiles will read
+                const uint64_t w_policy = t.once ? once_policy : reuse_policy;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                     unsigned char* sa = smem + stage * C::STAGE_BYTES;
@@ -368,27 +460,18 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
                     // the gather threads' copies complete on this barrier by their own arrivals
                     mbar_expect_tx(&full[stage], C::GATHER ? C::B_BYTES : C::STAGE_BYTES);
                     const int kx = (t.kb0 + kb) * kBK;
-                    if (SWAP) {
-                        if (p.w_tiles_hbm)
-                            bulk_g2s(sa, p.w_tiles_hbm + (((size_t)t.e * (p.w_rows / 128) + t.wt) * p.w_kb + (t.kb0 + kb)) * 16384,
-                                     16384, &full[stage]);
-                        else
-                            tma_load_2d(sa, &p.tm_w, &full[stage], kx, t.wrow0);
-                        tma_load_2d(sb, &p.tm_tok, &full[stage], kx, t.row0);
+                    if (!C::GATHER) tma_load_2d(sa, &p.tm_tok, &full[stage], kx, t.row0);
+                    if (EPI != 2) {
+                        bulk_g2s_hint(sb, w0, 16384, &full[stage], w_policy);
+                        bulk_g2s_hint(sb + 16384, w0 + w_next, 16384, &full[stage], w_policy);
+                        w0 += 16384;
                     } else {
-                        if (!C::GATHER) tma_load_2d(sa, &p.tm_tok, &full[stage], kx, t.row0);
-                        if (p.w_tiles_hbm) {
-                            const unsigned char* wt0 =
-                                p.w_tiles_hbm + (((size_t)t.e * (p.w_rows / 128) + 2 * t.wt) * p.w_kb + (t.kb0 + kb)) * 16384;
-                            bulk_g2s(sb, wt0, 16384, &full[stage]);
-                            bulk_g2s(sb + 16384, wt0 + (size_t)p.w_kb * 16384, 16384, &full[stage]);
-                        } else {
-                            tma_load_2d(sb, &p.tm_w, &full[stage], kx, t.wrow0);
-                        }
+                        tma_load_2d(sb, &p.tm_w, &full[stage], kx, t.wrow0);
                     }
                     ++issued;
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
+                if (!ok) break;
             }
             if (!ok) {
                 *abort_flag = 1;
@@ -402,13 +485,18 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(C::BM, C::BN);
+            constexpr uint32_t idesc = idesc_bf16(C::TOKTILE, C::WTILE);
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            RingCursor rc;
+            int tile = -1;
+            while (true) {
+                tile = C::DRAW ? ring_take(ring, rc) : rr_next(tile);
+                if (tile == -2) { ok = false; break; }
+                if (tile < 0) break;
                 if (!mbar_wait_or_abort(&acc_empty[acc], acc_phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * C::ACC_COLS);
@@ -447,7 +535,11 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            RingCursor rc;
+            while (true) {
+                const int tile = ring_take_warp(ring, rc, lane);
+                if (tile == -2) ok = false;
+                if (tile < 0) break;
                 const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
                 const __nv_bfloat16* src[8];
                 uint32_t nb[8];
@@ -470,6 +562,7 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
                     cp_async_arrive_noinc(&full[stage]);
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
+                if (!ok) break;
             }
             if (!ok) *abort_flag = 1;
             asm volatile("cp.async.wait_all;" ::: "memory");    // no copy in flight at exit
@@ -477,98 +570,60 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
     } else {
         // ------------------------------------------------ epilogue (warps 2..5)
         const int quad = warp & 3;                       // TMEM lane quadrant of this warp
-        unsigned char* stg = smem + STAGES * C::STAGE_BYTES + 256 + quad * 4096;
+        unsigned char* stg = smem + STAGES * C::STAGE_BYTES + C::BAR_BYTES + quad * 4096;
         int acc = 0;
         uint32_t acc_phase = 0;
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        RingCursor rc;
+        int tile = -1;
+        while (true) {
+            tile = C::DRAW ? ring_take_warp(ring, rc, lane) : rr_next(tile);
+            if (tile < 0) break;
             // the tile's rows and g_hat are read while its MMAs still run
             const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
-            const float gh = SWAP ? 0.f : wide_row_ghat<EPI>(p, t, quad * 32 + lane);
+            const float gh = wide_row_ghat<EPI>(p, t, quad * 32 + lane);
             bool ok = true;
             if (lane == 0) ok = mbar_wait_or_abort(&acc_full[acc], acc_phase, p.err, abort_flag);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * C::ACC_COLS);
-            if (SWAP) {
-                // lane = weight row (32 per warp), columns = TOKTILE (16) tokens
-                uint32_t r[16];
-                tmem_ld16(tbase, r);
-                tmem_ld_wait();
-                if (EPI == 0) {
-                    // rows: 16 gate then 16 up of FFN block (4 * wt + quad)
-                    const int j = (t.wt * 4 + quad) * 16 + (lane & 15);
-                    __nv_bfloat16* act = static_cast<__nv_bfloat16*>(p.out);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        const float v = __uint_as_float(r[c]);
-                        const float u = __shfl_xor_sync(0xffffffffu, v, 16);
-                        if (lane < 16 && c < t.nrows)
-                            act[(size_t)(t.row0 + c) * p.out_ld + j] = __float2bfloat16_rn(silu(v) * u);
-                    }
-                } else if (EPI == 1) {
-                    const int col = t.wt * C::WTILE + quad * 32 + lane;
-                    float* y = static_cast<float*>(p.out);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        if (c < t.nrows)
-                            y[(size_t)(t.row0 + c) * p.out_ld + col] = p.ghat[p.perm[t.row0 + c]] * __uint_as_float(r[c]);
-                    }
-                } else {
-                    // router logits: lane = expert, columns = tokens
-                    const int e = t.wt * C::WTILE + quad * 32 + lane;
-                    if (e < p.n_valid_cols) {
-                        float* z = static_cast<float*>(p.out);
-                        const float b = p.bias[e];
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            if (c < t.nrows) {
-                                float v = __uint_as_float(r[c]) + b;
-                                if (p.use_temp) v = v * p.inv_temp;
-                                z[(size_t)(t.row0 + c) * p.out_ld + e] = v;
-                            }
-                        }
-                    }
-                }
+            // lane = token row, columns = WTILE weight rows
+            if (EPI != 2) {
+                epilogue_wide<EPI>(p, t, tbase, quad * 32, lane, gh, stg);
             } else {
-                // lane = token row, columns = WTILE weight rows
                 const int row = quad * 32 + lane;
                 const bool valid = row < t.nrows;
                 const size_t orow = (size_t)(t.row0 + row);
-                if (EPI != 2) {
-                    epilogue_wide<EPI>(p, t, tbase, quad * 32, lane, gh, stg);
-                } else {
-                    // split-K: raw partial sums per slice (bias and temperature added by the consumer)
-                    float* z = static_cast<float*>(p.out) + (size_t)t.split * p.split_stride;
-                    const bool raw = splits > 1;
+                // split-K: raw partial sums per slice (bias and temperature added by the consumer)
+                float* z = static_cast<float*>(p.out) + (size_t)t.split * p.split_stride;
+                const bool raw = splits > 1;
 #pragma unroll 1
-                    for (int c0 = 0; c0 < C::WTILE; c0 += 16) {
-                        const int col0 = t.wt * C::WTILE + c0;
-                        if (col0 >= p.n_valid_cols) break;
-                        uint32_t r[16];
-                        tmem_ld16(tbase + c0, r);
-                        tmem_ld_wait();
-                        if (valid) {
-                            float v[16];
+                for (int c0 = 0; c0 < C::WTILE; c0 += 16) {
+                    const int col0 = t.wt * C::WTILE + c0;
+                    if (col0 >= p.n_valid_cols) break;
+                    uint32_t r[16];
+                    tmem_ld16(tbase + c0, r);
+                    tmem_ld_wait();
+                    if (valid) {
+                        float v[16];
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                const int col = min(col0 + i, p.n_valid_cols - 1);
-                                v[i] = __uint_as_float(r[i]);
-                                if (!raw) {
-                                    v[i] = v[i] + p.bias[col];
-                                    if (p.use_temp) v[i] = v[i] * p.inv_temp;
-                                }
+                        for (int i = 0; i < 16; ++i) {
+                            const int col = min(col0 + i, p.n_valid_cols - 1);
+                            v[i] = __uint_as_float(r[i]);
+                            if (!raw) {
+                                v[i] = v[i] + p.bias[col];
+                                if (p.use_temp) v[i] = v[i] * p.inv_temp;
                             }
-                            float* zr = z + orow * p.out_ld + col0;
-                            if (col0 + 16 <= p.n_valid_cols && (p.out_ld & 3) == 0) {
+                        }
+                        float* zr = z + orow * p.out_ld + col0;
+                        if (col0 + 16 <= p.n_valid_cols && (p.out_ld & 3) == 0) {
 #pragma unroll
-                                for (int i = 0; i < 16; i += 4)
-                                    *reinterpret_cast<float4*>(zr + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                            } else {
+                            for (int i = 0; i < 16; i += 4)
+                                *reinterpret_cast<float4*>(zr + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                        } else {
 #pragma unroll
-                                for (int i = 0; i < 16; ++i)
-                                    if (col0 + i < p.n_valid_cols) zr[i] = v[i];
-                            }
+                            for (int i = 0; i < 16; ++i)
+                                if (col0 + i < p.n_valid_cols) zr[i] = v[i];
                         }
                     }
                 }
@@ -588,8 +643,6 @@ __global__ void __launch_bounds__(TcCfg<SWAP, EPI, STAGES>::THREADS, 1) k_expert
                      "r"((uint32_t)C::TMEM_COLS));
     }
 }
-
-
 
 // ---------------------------------------------------------------- decode: both GEMMs in one launch
 //
@@ -1377,26 +1430,20 @@ cudaError_t launch_pair(const ace_layer* L, const TcParams& p, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, k_expert_pair<EPI>, p);
 }
 
-constexpr int kStagesSwap = 8;
 constexpr int kStagesWide = 4;
 
-template <bool SWAP, int EPI>
-constexpr int stages_for() { return SWAP ? kStagesSwap : kStagesWide; }
-
-template <bool SWAP, int EPI>
+template <int EPI>
 cudaError_t set_attr() {
-    constexpr int S = stages_for<SWAP, EPI>();
-    cudaError_t e = cudaFuncSetAttribute(k_expert_tc<SWAP, EPI, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         TcCfg<SWAP, EPI, S>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_expert_tc<EPI, kStagesWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         TcCfg<EPI, kStagesWide>::SMEM);
     if (e != cudaSuccess) return e;
-    return prefer_shared(k_expert_tc<SWAP, EPI, S>);
+    return prefer_shared(k_expert_tc<EPI, kStagesWide>);
 }
 
-template <bool SWAP, int EPI>
+template <int EPI>
 cudaError_t launch_gemm(const ace_layer* L, const TcParams& p, cudaStream_t s) {
-    constexpr int S = stages_for<SWAP, EPI>();
-    return launch_pdl(k_expert_tc<SWAP, EPI, S>, dim3(L->num_sms), dim3(TcCfg<SWAP, EPI, S>::THREADS),
-                      TcCfg<SWAP, EPI, S>::SMEM, s, p);
+    return launch_pdl(k_expert_tc<EPI, kStagesWide>, dim3(L->num_sms), dim3(TcCfg<EPI, kStagesWide>::THREADS),
+                      TcCfg<EPI, kStagesWide>::SMEM, s, p);
 }
 
 // Expert weights as tiles in HBM: block (e, t, kb) holds weight rows
@@ -1470,11 +1517,9 @@ cudaError_t tc_init(ace_layer* L) {
     if (!tc_supported(L)) return cudaSuccess;
     const ace_layer_desc& D = L->desc;
     cudaError_t e;
-    if ((e = set_attr<true, 0>()) != cudaSuccess) return e;
-    if ((e = set_attr<true, 1>()) != cudaSuccess) return e;
-    if ((e = set_attr<false, 0>()) != cudaSuccess) return e;
-    if ((e = set_attr<false, 1>()) != cudaSuccess) return e;
-    if ((e = set_attr<false, 2>()) != cudaSuccess) return e;
+    if ((e = set_attr<0>()) != cudaSuccess) return e;
+    if ((e = set_attr<1>()) != cudaSuccess) return e;
+    if ((e = set_attr<2>()) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_expert_decode<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   DecCfg<1>::SMEM)) != cudaSuccess)
         return e;
@@ -1511,7 +1556,6 @@ cudaError_t tc_init(ace_layer* L) {
     // tiled expert weights as rows of 64 bf16 (16 KB tiles = 128 rows), copied verbatim
     if ((e = make_map(&L->tcm.wgu_rows, L->w_gu, n * 2 * m * d / 64, 64, 128, false)) != cudaSuccess) return e;
     if ((e = make_map(&L->tcm.wd_rows, L->w_down, n * d * m / 64, 64, 128, false)) != cudaSuccess) return e;
-    if ((e = make_map(&L->tcm.tok1_small, L->ws.h_perm, rows, d, 16)) != cudaSuccess) return e;
     if ((e = make_map(&L->tcm.w_router_big, L->router_w, n_pad, d, 256)) != cudaSuccess) return e;
     return cudaSuccess;
 }
@@ -1549,7 +1593,7 @@ cudaError_t launch_router_tc(const ace_layer* L, int T, cudaStream_t s) {
     p.inv_temp = 1.0f / D.router_temp;
     p.use_temp = D.router_temp != 1.0f;
     p.n_valid_cols = D.n_experts;
-    return launch_gemm<false, 2>(L, p, s);
+    return launch_gemm<2>(L, p, s);
 }
 
 cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int T, ace_skip_ctl ctl, cudaStream_t s,
@@ -1612,7 +1656,7 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     }
     if (ev) ace::record_stage(ev[0], s);
     TcParams p1{};
-    p1.tm_tok = small ? L->tcm.tok1_small : L->tcm.tok1_big;
+    p1.tm_tok = L->tcm.tok1_big;
     p1.w_tiles_hbm = static_cast<const uint8_t*>(L->w_gu);
     p1.w_kb = d / kBK;
     p1.offsets = W.offsets;
@@ -1626,37 +1670,37 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     p1.h_src = static_cast<const __nv_bfloat16*>(W.h);
     p1.K = d;
     p1.w_rows = 2 * m;
-    p1.w_tiles = 2 * m / (small ? 128 : 256);
+    p1.w_tiles = 2 * m / 256;
+    p1.tile_next = W.meta + kMetaTile1;
     p1.out_ld = m;
     p1.err = W.err;
     if (pair) {
         TcParams q = p1;
         q.tm_w = L->tcm.wgu_rows;
-        q.w_tiles = 2 * m / 256;
         e = launch_pair<0>(L, q, s);
     } else {
-        e = small ? launch_gemm<true, 0>(L, p1, s) : launch_gemm<false, 0>(L, p1, s);
+        e = launch_gemm<0>(L, p1, s);
     }
     if (e != cudaSuccess) return e;
     if (ev) ace::record_stage(ev[1], s);
     TcParams p2 = p1;
-    p2.tm_tok = small ? L->tcm.tok2_small : L->tcm.tok2_big;
+    p2.tm_tok = L->tcm.tok2_big;
+    p2.tile_next = W.meta + kMetaTile2;
     p2.w_tiles_hbm = static_cast<const uint8_t*>(L->w_down);
     p2.w_kb = m / kBK;
-    // y per slot: fp32 rows for SWAP tiles; bf16 rows otherwise, written over
-    // h_perm, which GEMM 1 (complete before GEMM 2 reads anything) no longer needs
-    p2.out = small ? (void*)W.yslot : W.h_perm;
+    // y per slot: bf16 rows written over h_perm, which GEMM 1 (complete before
+    // GEMM 2 reads anything) no longer needs
+    p2.out = W.h_perm;
     p2.K = m;
     p2.w_rows = d;
-    p2.w_tiles = d / (small ? 128 : 256);
+    p2.w_tiles = d / 256;
     p2.out_ld = d;
     if (pair) {
         TcParams q = p2;
         q.tm_w = L->tcm.wd_rows;
-        q.w_tiles = d / 256;
         e = launch_pair<1>(L, q, s);
     } else {
-        e = small ? launch_gemm<true, 1>(L, p2, s) : launch_gemm<false, 1>(L, p2, s);
+        e = launch_gemm<1>(L, p2, s);
     }
     if (e != cudaSuccess) return e;
     if (ev) ace::record_stage(ev[2], s);
@@ -1665,12 +1709,7 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     const int32_t* sp = W.slot_pos;
     __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out);
     const int yr = T * k;                     // slot rows of this batch
-    if (small) {
-        const float* y = W.yslot;
-        e = k <= 8 ? launch_pdl(k_combine_bf16<float, 8>, grid, dim3(256), 0, s, y, sp, resid, o, T, d, k, yr, W.err)
-                   : launch_pdl(k_combine_bf16<float, kMaxTopK>, grid, dim3(256), 0, s, y, sp, resid, o, T, d, k, yr,
-                                W.err);
-    } else if (next) {
+    if (next) {
         const __nv_bfloat16* y = static_cast<const __nv_bfloat16*>(W.h_perm);
         e = k <= 8 ? launch_combine_norm<8>(y, sp, resid, o, next, T, d, k, yr, W.err, s)
                    : launch_combine_norm<kMaxTopK>(y, sp, resid, o, next, T, d, k, yr, W.err, s);

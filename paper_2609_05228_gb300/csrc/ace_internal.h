@@ -38,6 +38,8 @@ enum : int {
     kMetaSelWant = 11,     //   rank still wanted inside the first digit
     kMetaSelBelow = 12,    //   candidates below the first digit
     kMetaDecNext = 13,     // decode expert kernel: the next tile to take (zeroed by the routing)
+    kMetaTile1 = 14,       // prefill GEMM 1 / GEMM 2 (one CTA per tile): the next tile to take
+    kMetaTile2 = 15,       //   (zeroed by the compaction scan)
     kMetaCount = 16,
 };
 
@@ -81,7 +83,7 @@ struct Workspace {
 
 // Tensor maps of the tensor-core expert path (built once at create time).
 struct TcMaps {
-    CUtensorMap tok1_small, tok1_big;   // h_perm, boxes of 16 / 128 rows
+    CUtensorMap tok1_big;               // h_perm, boxes of 128 rows
     CUtensorMap tok2_small, tok2_big;   // act_bf16, boxes of 16 / 128 rows
     CUtensorMap h_rows_big, w_router_big;   // router GEMM (batches over 256 tokens): 128-row / 256-row boxes
     CUtensorMap wgu_rows, wd_rows;      // tiled W_gu / W_down as 128-B rows (CTA-pair kernel), no swizzle

@@ -962,6 +962,43 @@ __device__ __forceinline__ int block_exscan(int v, int* wtot, int& total) {
     return exc;
 }
 
+// The token-tile table of the one-CTA-per-tile prefill GEMMs (called by the
+// whole block after scan_counts_block and a barrier). An expert with one tile
+// streams its weights from HBM; of an expert with several, the first tile does
+// and the others find them in L2, bound by the MMAs. In expert order the large
+// experts run one after another with HBM nearly idle (8192 Zipf-routed tokens
+// on the large layer: 191 of 447 tiles), so the two kinds are interleaved in
+// proportion: with nM tiles in multi-tile experts (kept in expert order, so an
+// expert's tiles stay close and its weights stay in L2) and nS single-tile
+// experts, TT = nM + nS, entry p of the table is multi-tile where
+// floor((p + 1) nM / TT) steps up and single-tile elsewhere, which gives
+// element a of the first list entry ceil((a + 1) TT / nM) - 1 and element b of
+// the second entry floor(b TT / nS). The entry's last field marks the
+// single-tile experts (their weights give way first in L2).
+__device__ void fill_tile_table_mixed(const int32_t* offsets, const int32_t* dlist, const int32_t* tt_off,
+                                      const int32_t* meta, int tok_tile, int4* tt_tab, int n_exp, int tt_cap, int* err,
+                                      int* wtot) {
+    const int D = meta[kMetaDistinct], TT = meta[kMetaTokTiles];
+    const int per = (D + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int j0 = min((int)threadIdx.x * per, D), j1 = min(j0 + per, D);
+    int singles = 0;
+    for (int j = j0; j < j1; ++j) singles += tt_off[j + 1] - tt_off[j] == 1;
+    int nS;
+    int sb = block_exscan(singles, wtot, nS);            // single-tile experts before this thread's
+    const unsigned long long tt = TT, ns = nS, nm = TT - nS;
+    for (int j = j0; j < j1; ++j) {
+        const int e = dlist[j], base = tt_off[j], n = tt_off[j + 1] - base;
+        if (!ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) continue;
+        const int beg = offsets[e], cnt = offsets[e + 1] - beg;
+        for (int b = 0; b < n; ++b) {
+            const int pos = n == 1 ? (int)(sb * tt / ns) : (int)(((base - sb + b + 1) * tt + nm - 1) / nm) - 1;
+            if (!ACE_IDX_OK(pos >= 0 && pos < tt_cap, err)) break;
+            tt_tab[pos] = make_int4(e, beg + b * tok_tile, min(tok_tile, cnt - b * tok_tile), n == 1);
+        }
+        sb += n == 1;
+    }
+}
+
 // Block e: exclusive scan of counts[e][0 .. n_chunks) in place, row total to
 // offsets[e]. The last block (ticket in meta) turns the totals into
 // offsets[N+1], the distinct-expert list, the meta totals and the token-tile
@@ -1003,13 +1040,20 @@ __global__ void __launch_bounds__(kScanThreads) k_compact_scan(int n_exp, int n_
     if (tid == 0) s_last = atomicAdd(&meta[kMetaTicket], 1) == (int)gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
-    if (tid == 0) meta[kMetaTicket] = 0;
+    if (tid == 0) {
+        meta[kMetaTicket] = 0;
+        meta[kMetaTile1] = 0;             // the prefill GEMMs count up from zero
+        meta[kMetaTile2] = 0;
+    }
     __threadfence();
     for (int e = tid; e < n_exp; e += blockDim.x) cnt[e] = __ldcg(offsets + e);
     __syncthreads();
     scan_counts_block(cnt, n_exp, offsets, dlist, meta, nullptr, tok_tile, tt_off, wsum);
     __syncthreads();
-    fill_tile_table(offsets, dlist, tt_off, meta, tok_tile, tt_tab, n_exp, tt_cap, err);
+    if (tok_tile == 128)
+        fill_tile_table_mixed(offsets, dlist, tt_off, meta, tok_tile, tt_tab, n_exp, tt_cap, err, wtot);
+    else
+        fill_tile_table(offsets, dlist, tt_off, meta, tok_tile, tt_tab, n_exp, tt_cap, err);
 }
 
 __global__ void __launch_bounds__(kChunk) k_compact_place(int n_tokens, int k, int n_exp, int n_chunks,
