@@ -352,14 +352,12 @@ ace_status ace_route_decide_noalloc(const float* logits, int T, int n_experts, i
  *   gamma [d], router_w [N, d], w_gate / w_up [N, m, d], w_down [N, d, m]
  *                  device, bf16
  *   eps            the paper's epsilon (>= 0)
- *   tile_budget    device bytes for the repacked weight tiles (3 d m 2 bytes
- *                  per expert; experts are processed in chunks that fit, at
- *                  least one at a time); 0 = 1.5 GiB
+ *   tile_budget    not used: the weights are read in place
  *   gsp_out, rcr_out [N] host float32, written on success
- * Allocates its device scratch (the tiles plus O(N d) bytes) for the call
- * and frees it before returning; synchronises `stream`. Sums are taken in a
- * fixed order, so the result is the same bits on every run and for every
- * tile_budget.
+ * Allocates its device scratch (O(N d + N (d / 128)^2) bytes) for the call
+ * and frees it before returning; part of the work runs on a stream of its own,
+ * ordered within `stream`; synchronises `stream`. Sums are taken in a fixed
+ * order, so the result is the same bits on every run.
  * Errors: INVALID_ARG (NULL, non-positive size, eps < 0), UNSUPPORTED (shape),
  * OOM, CUDA, TIMEOUT (a bounded device wait ran out).
  */

@@ -1372,23 +1372,6 @@ cudaError_t get_encoder() {
     return cudaSuccess;
 }
 
-// 2-D bf16 map over [rows, cols] (row-major), box [box_rows, 64], 128-byte swizzle.
-// With swizzle == false the map copies rows verbatim (the tiled expert weights
-// are stored already swizzled).
-cudaError_t make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows,
-                     bool swizzle = true) {
-    cudaError_t e = get_encoder();
-    if (e != cudaSuccess) return e;
-    const cuuint64_t dims[2] = {cols, rows};
-    const cuuint64_t strides[1] = {cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 cudaError_t set_pair_attr(const void* k) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
     if (e != cudaSuccess) return e;
@@ -1482,6 +1465,23 @@ __global__ void __launch_bounds__(256) k_pack_tiles(const uint4* __restrict__ sr
 
 }  // namespace
 
+// 2-D bf16 map over [rows, cols] (row-major), box [box_rows, 64], 128-byte swizzle.
+// With swizzle == false the map copies rows verbatim (the tiled expert weights
+// are stored already swizzled).
+cudaError_t make_tensor_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                            bool swizzle) {
+    cudaError_t e = get_encoder();
+    if (e != cudaSuccess) return e;
+    const cuuint64_t dims[2] = {cols, rows};
+    const cuuint64_t strides[1] = {cols * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t tc_pack_weights(ace_layer* L, const void* w_gate, const void* w_up, const void* w_down, cudaStream_t s) {
     const ace_layer_desc& D = L->desc;
     k_pack_tiles<true><<<L->num_sms * 8, 256, 0, s>>>((const uint4*)w_gate, (const uint4*)w_up, (uint4*)L->w_gu,
@@ -1547,16 +1547,16 @@ cudaError_t tc_init(ace_layer* L) {
     const uint64_t n_pad = ((uint64_t)D.n_experts + 255) / 256 * 256;
     const uint64_t n = D.n_experts, d = D.hidden, m = D.ffn;
     // token maps: h_perm (GEMM 1) and act (GEMM 2), tiles of 16 / 128 rows
-    if ((e = make_map(&L->tcm.tok1_big, L->ws.h_perm, rows, d, 128)) != cudaSuccess) return e;
-    if ((e = make_map(&L->tcm.tok2_small, L->ws.act_bf16, rows, m, 16)) != cudaSuccess) return e;
-    if ((e = make_map(&L->tcm.tok2_big, L->ws.act_bf16, rows, m, 128)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.tok1_big, L->ws.h_perm, rows, d, 128, true)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.tok2_small, L->ws.act_bf16, rows, m, 16, true)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.tok2_big, L->ws.act_bf16, rows, m, 128, true)) != cudaSuccess) return e;
     // weight maps: W_gu [N * 2m, d] and W_down [N * d, m]
     // router: h [Tmax, d] in 128-row boxes, W_r [N, d] in 256-row boxes
-    if ((e = make_map(&L->tcm.h_rows_big, L->ws.h, h_rows, d, 128)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.h_rows_big, L->ws.h, h_rows, d, 128, true)) != cudaSuccess) return e;
     // tiled expert weights as rows of 64 bf16 (16 KB tiles = 128 rows), copied verbatim
-    if ((e = make_map(&L->tcm.wgu_rows, L->w_gu, n * 2 * m * d / 64, 64, 128, false)) != cudaSuccess) return e;
-    if ((e = make_map(&L->tcm.wd_rows, L->w_down, n * d * m / 64, 64, 128, false)) != cudaSuccess) return e;
-    if ((e = make_map(&L->tcm.w_router_big, L->router_w, n_pad, d, 256)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.wgu_rows, L->w_gu, n * 2 * m * d / 64, 64, 128, false)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.wd_rows, L->w_down, n * d * m / 64, 64, 128, false)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.w_router_big, L->router_w, n_pad, d, 256, true)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 

@@ -260,6 +260,10 @@ cudaError_t launch_experts_gemv(const ace_layer* L, const void* x, void* out, in
 constexpr int kNumStages = 7;
 
 // ---- tensor-core expert path (ace_expert_tc.cu) ----
+// 2-D bf16 tensor map over [rows, cols] (row-major), boxes of box_rows x 64,
+// 128-byte swizzle or none (rows copied verbatim).
+cudaError_t make_tensor_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                            bool swizzle);
 bool tc_supported(const ace_layer* L);
 int tc_token_tile(const ace_layer* L, int T, ace_skip_ctl ctl);
 bool tc_use_pair(const ace_layer* L, int T, ace_skip_ctl ctl);

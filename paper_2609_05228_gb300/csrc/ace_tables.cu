@@ -13,8 +13,12 @@
 // accumulators, sums them per row, scales row i by gamma_i^2 (so Gamma is
 // applied exactly, not rounded into a bf16 operand) and writes one fp64
 // partial per (tile, warp). The nn.Linear layouts give W_p[i, r] =
-// w_p[e][r][i] (the A operand, transposed into K-major tiles here) and
-// W_down[r, j] = w_down[e][j][r] (the B operand, K-major as stored).
+// w_p[e][r][i] (the A operand, M-major: TMA loads 64 x 64 boxes of the weights
+// as stored and the instruction descriptor says so) and W_down[r, j] =
+// w_down[e][j][r] (the B operand, K-major as stored). The weights are read in
+// place: repacking them into K-major tiles first took 0.53 ms of kernels and
+// most of a 1.2 GB scratch allocation's 1 ms at d = 2048, N = 128, m = 768 (a
+// call took 2.71 ms, 1.47 without).
 //
 // RCR (Algorithm 3; Eqs. rcr_centered_router, rcr_direction_prototype,
 // rcr_raw_amplification, rcr_layer_normalization): centred router rows
@@ -45,7 +49,6 @@ constexpr int kTabA = 128 * kBK * 2;            // 16 KB: 128 rows i x 64 r
 constexpr int kTabB = 256 * kBK * 2;            // 32 KB: 256 rows j x 64 r
 constexpr int kTabStage = kTabA + kTabB;
 constexpr int kTabSmem = kTabStages * kTabStage + 1024 + 256;
-constexpr int kTile = 16384;                    // bytes of one 128 x 64 bf16 tile
 
 // Fixed-order block sum of one double per thread (blockDim.x = 256).
 __device__ __forceinline__ double block_sum_256(double v, double* sh) {
@@ -60,97 +63,14 @@ __device__ __forceinline__ double block_sum_256(double v, double* sh) {
     return t;   // valid in thread 0
 }
 
-// ---------------------------------------------------------------- packing
-//
-// Tiles: block (e, t, kb) holds rows [128 t, 128 t + 128) and K columns
-// [64 kb, 64 kb + 64) as 128 rows of 128 bytes; the 16-byte chunk c of row r
-// sits at chunk position c ^ (r & 7) (the 128-byte swizzle that the
-// tcgen05 shared-memory descriptor expects). Layout [e][t][kb].
-
-// B operand: w_down[e] is [d][m] with K = m contiguous, so tiles are gathers.
-__global__ void __launch_bounds__(256) k_pack_rows(const uint4* __restrict__ src, uint4* __restrict__ dst, int n_e,
-                                                   int rows, int K) {
-    const int cv = K / 8, kbs = K / 64, ts = rows / 128;
-    const long long total = (long long)n_e * rows * cv;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long blk = q >> 10;
-        const int w = (int)(q & 1023);
-        const int r = w >> 3, c = (w & 7) ^ (r & 7);
-        const int kb = (int)(blk % kbs);
-        const long long et = blk / kbs;
-        const int t = (int)(et % ts);
-        const long long e = et / ts;
-        dst[q] = src[(e * rows + t * 128 + r) * cv + kb * 8 + c];
-    }
-}
-
-// A operand: w_p[e] is [m][d] (K = m is the slow index), so each block
-// transposes a 64 (r) x 128 (i) sub-matrix into one tile through shared
-// memory: coalesced 16-byte reads into a row-major staging buffer; each warp
-// then builds the 16-byte chunks of 32 consecutive tile rows i (one logical
-// chunk c at a time, conflict-free column reads) and stores them at their
-// swizzled positions in a second buffer (8 consecutive rows hit 8 distinct
-// 16-byte bank groups); the finished tile leaves in coalesced 16-byte writes.
-// The same pass accumulates the block's share of ||Gamma W_p||_F^2 =
-// sum_{r,i} gamma_i^2 W_p[i, r]^2 (one fp64 partial per block, fixed order).
-constexpr int kTrLd = 128 + 2;                  // staging row (bf16): 65 words, odd
-
-__global__ void __launch_bounds__(256) k_pack_transposed(const __nv_bfloat16* __restrict__ src,
-                                                         const float* __restrict__ gamma2,
-                                                         uint4* __restrict__ dst, double* __restrict__ norm_part,
-                                                         int d, int m) {
-    __shared__ __align__(16) __nv_bfloat16 buf[64 * kTrLd];
-    __shared__ __align__(16) uint4 tile[1024];
-    __shared__ double sh[8];
-    const int kbs = m / 64, ts = d / 128;
-    const int kb = blockIdx.x % kbs;
-    const int t = (blockIdx.x / kbs) % ts;
-    const long long e = blockIdx.x / ((long long)kbs * ts);
-    const __nv_bfloat16* s = src + (e * m + (long long)kb * 64) * d + (long long)t * 128;
-    double acc = 0.0;
-    for (int q = threadIdx.x; q < 64 * 16; q += 256) {
-        const int r = q >> 4, c = q & 15;          // 16 chunks of 8 along i
-        const uint4 v = *reinterpret_cast<const uint4*>(s + (long long)r * d + c * 8);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        float f[8];
-        Vec16<__nv_bfloat16>::to_float(v, f);
-        float sq = 0.f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sq = fmaf(gamma2[t * 128 + c * 8 + j] * f[j], f[j], sq);
-        acc += (double)sq;
-        uint32_t* row = reinterpret_cast<uint32_t*>(&buf[r * kTrLd + c * 8]);   // 4-byte aligned (kTrLd even)
-#pragma unroll
-        for (int h = 0; h < 4; ++h) row[h] = w[h];
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int job = warp; job < 32; job += 8) {      // 4 groups of 32 rows x 8 logical chunks
-        const int i = (job & 3) * 32 + lane, c = job >> 2;
-        uint32_t w[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const uint32_t lo = __bfloat16_as_ushort(buf[(8 * c + 2 * h) * kTrLd + i]);
-            const uint32_t hi = __bfloat16_as_ushort(buf[(8 * c + 2 * h + 1) * kTrLd + i]);
-            w[h] = lo | (hi << 16);
-        }
-        tile[i * 8 + (c ^ (i & 7))] = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-    __syncthreads();
-    uint4* out = dst + (long long)blockIdx.x * 1024;
-    for (int q = threadIdx.x; q < 1024; q += 256) out[q] = tile[q];
-    const double tot = block_sum_256(acc, sh);
-    if (threadIdx.x == 0) norm_part[blockIdx.x] = tot;
-}
-
 // ---------------------------------------------------------------- GSP: Frobenius norms of the products
 
 struct FrobParams {
-    const uint8_t* a_tiles[2];   // gate, up: [n_e][d/128][m/64] tiles (rows i, K = r)
-    const uint8_t* b_tiles;      // w_down:   [n_e][d/128][m/64] tiles (rows j, K = r)
+    CUtensorMap tm_a[2];         // gate, up as [N * m rows r, d columns i]: boxes of 64 r x 64 i
+    CUtensorMap tm_b;            // w_down as [N * d rows j, m columns r]: boxes of 256 j x 64 r
     const float* gamma2;         // [d] gamma_i^2 (exact in fp32 for bf16 gamma)
-    double* partial;             // [N][2][d/128 * d/256][4], indexed by the global expert
-    int e0, n_e, d, m;
+    double* partial;             // [N][2][d/128 * d/256][4]
+    int n_e, d, m;
     int* err;
 };
 
@@ -172,9 +92,23 @@ __device__ __forceinline__ FrobItem frob_item(const FrobParams& p, int item) {
     return it;
 }
 
+// Shared-memory descriptor of an M-major operand tile in the 128-byte swizzle:
+// 64-element M blocks of 128-byte rows, one row per K index; 8 rows (1024
+// bytes) to the next group of K indices, 64 rows (8 KB) to the next M block.
+__device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFF);          // start address
+    d |= (uint64_t)(8192 >> 4) << 16;               // leading byte offset: next 64-element M block
+    d |= (uint64_t)(1024 >> 4) << 32;               // stride byte offset: next 8 K indices
+    d |= (uint64_t)1 << 46;                         // descriptor version
+    d |= (uint64_t)2 << 61;                         // 128-byte swizzle
+    return d;
+}
+
 // 128 x 256 output tiles of C = A B^T, K = m, persistent over the items;
-// warp 0 loads (bulk copies of pre-swizzled tiles), warp 1 issues the MMAs,
+// warp 0 loads (TMA boxes of the weights as stored), warp 1 issues the MMAs,
 // warps 2..5 reduce the accumulators. Two 256-column accumulator buffers.
+// Bound by the tensor pipe under the power limit.
 __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_constant__ FrobParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -217,16 +151,14 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
             long long issued = 0;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const FrobItem it = frob_item(p, item);
-                const uint8_t* a = p.a_tiles[it.path] + ((size_t)it.el * ti_n + it.ti) * kblocks * kTile;
-                const uint8_t* b0 = p.b_tiles + ((size_t)it.el * ti_n + 2 * it.tj) * kblocks * kTile;
-                const uint8_t* b1 = b0 + (size_t)kblocks * kTile;
+                const int a_row = it.el * p.m, b_row = it.el * p.d + it.tj * 256;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, p.err) || *abort_flag) { ok = false; break; }
                     unsigned char* sa = smem + stage * kTabStage;
                     mbar_expect_tx(&full[stage], kTabStage);
-                    bulk_g2s(sa, a + (size_t)kb * kTile, kTile, &full[stage]);
-                    bulk_g2s(sa + kTabA, b0 + (size_t)kb * kTile, kTile, &full[stage]);
-                    bulk_g2s(sa + kTabA + kTile, b1 + (size_t)kb * kTile, kTile, &full[stage]);
+                    tma_load_2d(sa, &p.tm_a[it.path], &full[stage], it.ti * 128, a_row + kb * kBK);
+                    tma_load_2d(sa + kTabA / 2, &p.tm_a[it.path], &full[stage], it.ti * 128 + 64, a_row + kb * kBK);
+                    tma_load_2d(sa + kTabA, &p.tm_b, &full[stage], kb * kBK, b_row);
                     ++issued;
                     if (++stage == kTabStages) { stage = 0; phase ^= 1u; }
                 }
@@ -240,7 +172,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(128, 256);
+            constexpr uint32_t idesc = idesc_bf16(128, 256) | (1u << 15);   // A is M-major
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -255,10 +187,11 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
                     tc_fence_after();
                     const uint32_t a_addr = smem_u32(smem + stage * kTabStage);
                     const uint32_t b_addr = a_addr + kTabA;
+                    // a K step of 16: 16 rows of A (2 KB), 32 bytes of B (addresses in units of 16 bytes)
+                    const uint64_t ad = smem_desc_sw128_mn(a_addr), bd = smem_desc_sw128(b_addr);
 #pragma unroll
                     for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                        mma_bf16(d_tmem, smem_desc_sw128(a_addr + kk * kUmmaK * 2),
-                                 smem_desc_sw128(b_addr + kk * kUmmaK * 2), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                        mma_bf16(d_tmem, ad + 128 * kk, bd + 2 * kk, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                     mma_commit(&empty[stage]);
                     if (++stage == kTabStages) { stage = 0; phase ^= 1u; }
                 }
@@ -307,7 +240,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
             for (int o = 16; o > 0; o >>= 1) row += __shfl_xor_sync(0xffffffffu, row, o);
             if (lane == 0) {
                 const size_t tile = (size_t)it.tj * ti_n + it.ti;
-                p.partial[(((size_t)(p.e0 + it.el) * 2 + it.path) * ti_n * tj_n + tile) * 4 + quad] = row;
+                p.partial[(((size_t)it.el * 2 + it.path) * ti_n * tj_n + tile) * 4 + quad] = row;
             }
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -359,34 +292,56 @@ __global__ void __launch_bounds__(256) k_rcr_proto(const __nv_bfloat16* __restri
 }
 
 // act_e[j] = SiLU(x_e . W_gate[e, j]) * (x_e . W_up[e, j]); grid (m / 64, N),
-// each warp 8 rows j, one input row in shared memory.
-__global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w_gate,
+// each warp 8 rows j, the input row and gamma^2 in shared memory. The rows
+// pass here anyway, so the block also sums its share of ||Gamma W_gate||_F^2
+// and ||Gamma W_up||_F^2: gamma_i^2 w^2 over 8 elements in fp32, those sums in
+// fp64, lanes and warps in a fixed order; one partial per block and path in
+// norms[path][e][block].
+__global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x, const float* __restrict__ gamma2,
+                                                    const __nv_bfloat16* __restrict__ w_gate,
                                                     const __nv_bfloat16* __restrict__ w_up, int d, int m,
-                                                    float* __restrict__ act) {
+                                                    float* __restrict__ act, double* __restrict__ norms) {
     extern __shared__ __align__(16) float xs[];
+    __shared__ double sh[8];
+    float* gs = xs + d;
     const long long e = blockIdx.y;
-    for (int i = threadIdx.x; i < d; i += 256) xs[i] = x[e * d + i];
+    for (int i = threadIdx.x; i < d; i += 256) {
+        xs[i] = x[e * d + i];
+        gs[i] = gamma2[i];
+    }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cv = d / 8;
+    double ng = 0.0, nu = 0.0;
     for (int t = 0; t < 8; ++t) {
         const int j = blockIdx.x * 64 + warp * 8 + t;
         const uint4* g = reinterpret_cast<const uint4*>(w_gate + (e * m + j) * (long long)d);
         const uint4* u = reinterpret_cast<const uint4*>(w_up + (e * m + j) * (long long)d);
         float sg = 0.f, su = 0.f;
+#pragma unroll 4
         for (int q = lane; q < cv; q += 32) {
             float fg[8], fu[8];
             Vec16<__nv_bfloat16>::to_float(ld_stream(g + q), fg);
             Vec16<__nv_bfloat16>::to_float(ld_stream(u + q), fu);
+            float qg = 0.f, qu = 0.f;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 sg = fmaf(fg[k], xs[q * 8 + k], sg);
                 su = fmaf(fu[k], xs[q * 8 + k], su);
+                qg = fmaf(gs[q * 8 + k] * fg[k], fg[k], qg);
+                qu = fmaf(gs[q * 8 + k] * fu[k], fu[k], qu);
             }
+            ng += (double)qg;
+            nu += (double)qu;
         }
         sg = warp_sum(sg);
         su = warp_sum(su);
         if (lane == 0) act[e * m + j] = sg / (1.0f + expf(-sg)) * su;
+    }
+    const double tg = block_sum_256(ng, sh), tu = block_sum_256(nu, sh);
+    if (threadIdx.x == 0) {
+        norms[e * gridDim.x + blockIdx.x] = tg;
+        norms[((long long)gridDim.y + e) * gridDim.x + blockIdx.x] = tu;
     }
 }
 
@@ -511,19 +466,12 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return tab_fail(ACE_ERR_CUDA, std::string("ace_offline_tables_device: ") + cudaGetErrorString(e));
 
-    // experts per chunk: three tile copies (A gate, A up, B) within the budget
-    const size_t per_expert = 3ull * d * m * 2;
-    const size_t budget = tile_budget ? tile_budget : (1536ull << 20);
-    long long chunk_ll = (long long)(budget / per_expert);
-    int chunk = chunk_ll > N ? N : (int)chunk_ll;
-    chunk = chunk < 1 ? 1 : chunk;
+    (void)tile_budget;          // the weights are read in place
     const int ti_n = d / 128, tj_n = d / 256, frob_per = ti_n * tj_n * 4, rcr_per = d / 64;
-    const int norm_per = ti_n * (m / 64);        // k_pack_transposed blocks per expert
+    const int norm_per = m / 64;                 // k_rcr_gateup blocks per expert
 
-    const size_t tiles_bytes = (size_t)chunk * d * m * 2;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
-    const size_t o_a0 = take(tiles_bytes), o_a1 = take(tiles_bytes), o_b = take(tiles_bytes);
     const size_t o_frob = take((size_t)N * 2 * frob_per * 8), o_norm = take((size_t)N * 2 * norm_per * 8);
     const size_t o_raw = take((size_t)N * 5 * 8);
     const size_t o_mean = take((size_t)d * 8), o_x = take((size_t)N * d * 4), o_qn = take((size_t)N * 8);
@@ -540,6 +488,9 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
     int* err = reinterpret_cast<int*>(base + o_err);
     float* out = reinterpret_cast<float*>(base + o_out);
     int herr = 0;
+    // the RCR chain (HBM-bound) runs beside the GSP GEMM (tensor-bound) on a stream of the call
+    cudaStream_t s2 = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
 #define TAB_CK(call)                                                                                      \
     do {                                                                                                  \
         cudaError_t e_ = (call);                                                                          \
@@ -548,54 +499,48 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
             goto done;                                                                                    \
         }                                                                                                 \
     } while (0)
+    FrobParams p{};
     TAB_CK(cudaFuncSetAttribute(k_gsp_frob, cudaFuncAttributeMaxDynamicSharedMemorySize, kTabSmem));
-    TAB_CK(ace::raise_smem_limit(k_rcr_gateup, d * 4));
+    TAB_CK(ace::raise_smem_limit(k_rcr_gateup, d * 8));
     TAB_CK(ace::raise_smem_limit(k_rcr_down, m * 4));
+    TAB_CK(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking));
+    TAB_CK(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
+    TAB_CK(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
+    TAB_CK(make_tensor_map(&p.tm_a[0], wg, (uint64_t)N * m, d, 64, true));
+    TAB_CK(make_tensor_map(&p.tm_a[1], wu, (uint64_t)N * m, d, 64, true));
+    TAB_CK(make_tensor_map(&p.tm_b, wd, (uint64_t)N * d, m, 256, true));
     TAB_CK(cudaMemsetAsync(err, 0, 4, s));
     k_gamma2<<<(d + 255) / 256, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(gamma), g2, d);
     TAB_CK(cudaGetLastError());
-    for (int e0 = 0; e0 < N; e0 += chunk) {
-        const int n_e = N - e0 < chunk ? N - e0 : chunk;
-        const size_t eo = (size_t)e0 * m * d;
-        const int tblocks = n_e * ti_n * (m / 64);
-        double* norm = reinterpret_cast<double*>(base + o_norm);   // [path][e][norm_per]
-        k_pack_transposed<<<tblocks, 256, 0, s>>>(wg + eo, g2, reinterpret_cast<uint4*>(base + o_a0),
-                                                  norm + (size_t)e0 * norm_per, d, m);
-        TAB_CK(cudaGetLastError());
-        k_pack_transposed<<<tblocks, 256, 0, s>>>(wu + eo, g2, reinterpret_cast<uint4*>(base + o_a1),
-                                                  norm + ((size_t)N + e0) * norm_per, d, m);
-        TAB_CK(cudaGetLastError());
-        k_pack_rows<<<sms * 8, 256, 0, s>>>(reinterpret_cast<const uint4*>(wd + eo), reinterpret_cast<uint4*>(base + o_b),
-                                            n_e, d, m);
-        TAB_CK(cudaGetLastError());
-        FrobParams p{};
-        p.a_tiles[0] = base + o_a0;
-        p.a_tiles[1] = base + o_a1;
-        p.b_tiles = base + o_b;
-        p.gamma2 = g2;
-        p.partial = reinterpret_cast<double*>(base + o_frob);
-        p.e0 = e0;
-        p.n_e = n_e;
-        p.d = d;
-        p.m = m;
-        p.err = err;
-        const int items = n_e * 2 * ti_n * tj_n;
-        k_gsp_frob<<<items < sms ? items : sms, kTabThreads, kTabSmem, s>>>(p);
+    TAB_CK(cudaEventRecord(fork, s));
+    TAB_CK(cudaStreamWaitEvent(s2, fork, 0));
+    p.gamma2 = g2;
+    p.partial = reinterpret_cast<double*>(base + o_frob);
+    p.n_e = N;
+    p.d = d;
+    p.m = m;
+    p.err = err;
+    {
+        const long long items = (long long)N * 2 * ti_n * tj_n;
+        k_gsp_frob<<<items < sms ? (int)items : sms, kTabThreads, kTabSmem, s>>>(p);
         TAB_CK(cudaGetLastError());
     }
-    k_rcr_colmean<<<(d + 255) / 256, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(router_w), N, d,
-                                                  reinterpret_cast<double*>(base + o_mean));
+    k_rcr_colmean<<<(d + 255) / 256, 256, 0, s2>>>(static_cast<const __nv_bfloat16*>(router_w), N, d,
+                                                   reinterpret_cast<double*>(base + o_mean));
     TAB_CK(cudaGetLastError());
-    k_rcr_proto<<<N, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(router_w), reinterpret_cast<double*>(base + o_mean),
-                                  static_cast<const __nv_bfloat16*>(gamma), rcr_apply_gamma, d, eps,
-                                  reinterpret_cast<float*>(base + o_x), reinterpret_cast<double*>(base + o_qn));
+    k_rcr_proto<<<N, 256, 0, s2>>>(static_cast<const __nv_bfloat16*>(router_w), reinterpret_cast<double*>(base + o_mean),
+                                   static_cast<const __nv_bfloat16*>(gamma), rcr_apply_gamma, d, eps,
+                                   reinterpret_cast<float*>(base + o_x), reinterpret_cast<double*>(base + o_qn));
     TAB_CK(cudaGetLastError());
-    k_rcr_gateup<<<dim3(m / 64, N), 256, d * 4, s>>>(reinterpret_cast<const float*>(base + o_x), wg, wu, d, m,
-                                                     reinterpret_cast<float*>(base + o_act));
+    k_rcr_gateup<<<dim3(m / 64, N), 256, d * 8, s2>>>(reinterpret_cast<const float*>(base + o_x), g2, wg, wu, d, m,
+                                                      reinterpret_cast<float*>(base + o_act),
+                                                      reinterpret_cast<double*>(base + o_norm));
     TAB_CK(cudaGetLastError());
-    k_rcr_down<<<dim3(d / 64, N), 256, m * 4, s>>>(reinterpret_cast<const float*>(base + o_act), wd, d, m,
-                                                   reinterpret_cast<double*>(base + o_rcr));
+    k_rcr_down<<<dim3(d / 64, N), 256, m * 4, s2>>>(reinterpret_cast<const float*>(base + o_act), wd, d, m,
+                                                    reinterpret_cast<double*>(base + o_rcr));
     TAB_CK(cudaGetLastError());
+    TAB_CK(cudaEventRecord(join, s2));
+    TAB_CK(cudaStreamWaitEvent(s, join, 0));
     k_tables_reduce<<<N, 256, 0, s>>>(reinterpret_cast<const double*>(base + o_frob), frob_per,
                                       reinterpret_cast<const double*>(base + o_norm), norm_per,
                                       reinterpret_cast<const double*>(base + o_rcr), rcr_per, N,
@@ -612,6 +557,12 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
 #undef TAB_CK
 done:
     cudaStreamSynchronize(s);
+    if (s2) {
+        cudaStreamSynchronize(s2);
+        cudaStreamDestroy(s2);
+    }
+    if (fork) cudaEventDestroy(fork);
+    if (join) cudaEventDestroy(join);
     cudaFree(base);
     return st;
 }
