@@ -3,10 +3,13 @@
 // combine (Eq. ace_sparse_output).
 //
 // Work items are (distinct retained expert, slice of weight rows); the
-// compaction's last block sizes the slices so that there are about four
-// items per SM. Each item streams its weight rows once per chunk of up to
-// kGemvTokenChunk tokens routed to that expert, with 16-byte non-caching
-// loads; the tokens' activations sit in shared memory.
+// blocks take equal shares of the weight rows. Each item streams its weight
+// rows once per chunk of up to TC tokens routed to that expert, with 16-byte
+// non-caching loads; the tokens' activations sit in shared memory, and a
+// warp's first weights are on their way before it stages them. Small layers
+// are bound by that chain of dependent loads and by the launches (PDL), so a
+// chunk is 16 tokens where they fit (an expert's tokens in one pass instead of
+// two): 64 tokens on the (256, 16 experts, top-4, 128) fp32 layer.
 //   gate/up: act[r, j] = SiLU(h_t . W_gate[e, j]) * (h_t . W_up[e, j])
 //   down:    y[r, c]   = g_hat(r) * (act[r] . W_down[e, c])
 //   combine: out[t, c] = sum over t's kept slots, in rank order, of y[r, c]
@@ -17,8 +20,6 @@
 
 namespace ace {
 namespace {
-
-constexpr int kTC = kGemvTokenChunk;
 
 __device__ __forceinline__ float silu(float u) { return u / (1.0f + expf(-u)); }
 
@@ -31,7 +32,7 @@ __device__ __forceinline__ void block_range(long long total, long long& lo, long
 
 // gate/up: one warp per row pair (W_gate[e, j], W_up[e, j]); each lane issues
 // up to kCh 16-byte loads of each row before the dot products.
-template <typename T>
+template <typename T, int kTC>
 __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, const T* __restrict__ w_gate,
                                                      const T* __restrict__ w_up,
                                                      const int32_t* __restrict__ offsets,
@@ -39,7 +40,8 @@ __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, co
                                                      const int32_t* __restrict__ perm,
                                                      const int32_t* __restrict__ meta,
                                                      float* __restrict__ act, int d, int m, int k) {
-    constexpr int kCh = 8;
+    constexpr int kCh = kTC <= 8 ? 8 : 4;
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint4* hs = reinterpret_cast<uint4*>(smem_raw);     // [kTC][d / V] vectors
     constexpr int V = Vec16<T>::N;
@@ -55,6 +57,20 @@ __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, co
         const int r0 = offsets[e], ne = offsets[e + 1] - r0;
         for (int tc0 = 0; tc0 < ne; tc0 += kTC) {
             const int ntc = min(kTC, ne - tc0);
+            // the first row pair's leading chunks load while the tokens are staged
+            uint4 vg[kCh], vu[kCh];
+            const auto load = [&](int j, int c0) {
+                const uint4* wg = reinterpret_cast<const uint4*>(w_gate + ((size_t)e * m + j) * d);
+                const uint4* wu = reinterpret_cast<const uint4*>(w_up + ((size_t)e * m + j) * d);
+#pragma unroll
+                for (int i = 0; i < kCh; ++i) {
+                    const int c = c0 + lane + 32 * i;
+                    const bool ok = c < nvec;
+                    vg[i] = ok ? ld_stream(wg + c) : make_uint4(0, 0, 0, 0);
+                    vu[i] = ok ? ld_stream(wu + c) : make_uint4(0, 0, 0, 0);
+                }
+            };
+            if (rb + warp < re) load(rb + warp, 0);
             __syncthreads();
             for (int i = threadIdx.x; i < ntc * nvec; i += blockDim.x) {
                 const int q = i / nvec, c = i % nvec;
@@ -63,20 +79,11 @@ __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, co
             }
             __syncthreads();
             for (int j = rb + warp; j < re; j += nwarps) {
-                const uint4* wg = reinterpret_cast<const uint4*>(w_gate + ((size_t)e * m + j) * d);
-                const uint4* wu = reinterpret_cast<const uint4*>(w_up + ((size_t)e * m + j) * d);
                 float ag[kTC], au[kTC];
 #pragma unroll
                 for (int q = 0; q < kTC; ++q) { ag[q] = 0.f; au[q] = 0.f; }
                 for (int c0 = 0; c0 < nvec; c0 += 32 * kCh) {
-                    uint4 vg[kCh], vu[kCh];
-#pragma unroll
-                    for (int i = 0; i < kCh; ++i) {
-                        const int c = c0 + lane + 32 * i;
-                        const bool ok = c < nvec;
-                        vg[i] = ok ? ld_stream(wg + c) : make_uint4(0, 0, 0, 0);
-                        vu[i] = ok ? ld_stream(wu + c) : make_uint4(0, 0, 0, 0);
-                    }
+                    if (j != rb + warp || c0 != 0) load(j, c0);
 #pragma unroll
                     for (int i = 0; i < kCh; ++i) {
                         const int c = c0 + lane + 32 * i;
@@ -114,7 +121,7 @@ __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, co
 
 // down: one warp per 4 rows W_down[e, c..c+3] (each m long); up to kCh
 // 16-byte loads per row and lane are in flight before the dot products.
-template <typename T>
+template <typename T, int kTC>
 __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act, const T* __restrict__ w_down,
                                                    const float* __restrict__ ghat,
                                                    const int32_t* __restrict__ offsets,
@@ -122,8 +129,9 @@ __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act
                                                    const int32_t* __restrict__ perm,
                                                    const int32_t* __restrict__ meta,
                                                    float* __restrict__ yslot, int d, int m) {
-    constexpr int kCh = 4;
+    constexpr int kCh = kTC <= 8 ? 4 : 2;
     constexpr int kRows = 4;
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* as = reinterpret_cast<float*>(smem_raw);      // [kTC][m]
     __shared__ float gs[kTC];
@@ -140,6 +148,21 @@ __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act
         const int r0 = offsets[e], ne = offsets[e + 1] - r0;
         for (int tc0 = 0; tc0 < ne; tc0 += kTC) {
             const int ntc = min(kTC, ne - tc0);
+            // the first rows' leading chunks load while the activations are staged
+            uint4 wv[kRows][kCh];
+            const auto load = [&](int c, int v0) {
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) {
+                    const uint4* wd = reinterpret_cast<const uint4*>(w_down + ((size_t)e * d + c + r) * m);
+#pragma unroll
+                    for (int i = 0; i < kCh; ++i) {
+                        const int v = v0 + lane + 32 * i;
+                        wv[r][i] = (c + r < re && v < nvec) ? ld_stream(wd + v) : make_uint4(0, 0, 0, 0);
+                    }
+                }
+            };
+            const int first = rb + warp * kRows;
+            if (first < re) load(first, 0);
             __syncthreads();
             for (int i = threadIdx.x; i < ntc * (m / 4); i += blockDim.x) {
                 const int q = i / (m / 4), c = i % (m / 4);
@@ -147,23 +170,14 @@ __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act
             }
             if (threadIdx.x < kTC) gs[threadIdx.x] = threadIdx.x < ntc ? ghat[perm[r0 + tc0 + threadIdx.x]] : 0.f;
             __syncthreads();
-            for (int c = rb + warp * kRows; c < re; c += nwarps * kRows) {
+            for (int c = first; c < re; c += nwarps * kRows) {
                 float acc[kRows][kTC];
 #pragma unroll
                 for (int r = 0; r < kRows; ++r)
 #pragma unroll
                     for (int q = 0; q < kTC; ++q) acc[r][q] = 0.f;
                 for (int v0 = 0; v0 < nvec; v0 += 32 * kCh) {
-                    uint4 wv[kRows][kCh];
-#pragma unroll
-                    for (int r = 0; r < kRows; ++r) {
-                        const uint4* wd = reinterpret_cast<const uint4*>(w_down + ((size_t)e * d + c + r) * m);
-#pragma unroll
-                        for (int i = 0; i < kCh; ++i) {
-                            const int v = v0 + lane + 32 * i;
-                            wv[r][i] = (c + r < re && v < nvec) ? ld_stream(wd + v) : make_uint4(0, 0, 0, 0);
-                        }
-                    }
+                    if (c != first || v0 != 0) load(c, v0);
 #pragma unroll
                     for (int i = 0; i < kCh; ++i) {
                         const int v = v0 + lane + 32 * i;
@@ -205,22 +219,30 @@ __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act
     }
 }
 
-// out[t, c] = sum_{i kept, rank order} y[slot_pos[t*k+i], c]
-template <typename T>
+// out[t, c] = (x[t, c] +) sum_{i kept, rank order} y[slot_pos[t*k+i], c]; a
+// token's row indices are read together, then its rows, then the sum.
+template <typename T, int KMAX>
 __global__ void __launch_bounds__(256) k_combine(const float* __restrict__ yslot,
                                                  const int32_t* __restrict__ slot_pos, const T* __restrict__ resid,
                                                  T* __restrict__ out, int n_tokens, int d, int k) {
+    pdl_wait();
     const int nq = d / 4;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)n_tokens * nq) return;
     const int t = (int)(idx / nq), c4 = (int)(idx % nq);
+    int r[KMAX];
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i) r[i] = i < k ? __ldg(slot_pos + (size_t)t * k + i) : -1;
+    float4 y[KMAX];
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+        if (r[i] >= 0) y[i] = reinterpret_cast<const float4*>(yslot + (size_t)r[i] * d)[c4];
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = 0; i < k; ++i) {
-        const int r = slot_pos[(size_t)t * k + i];
-        if (r < 0) continue;
-        const float4 y = reinterpret_cast<const float4*>(yslot + (size_t)r * d)[c4];
-        acc.x += y.x; acc.y += y.y; acc.z += y.z; acc.w += y.w;
-    }
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+        if (r[i] >= 0) {
+            acc.x += y[i].x; acc.y += y[i].y; acc.z += y[i].z; acc.w += y[i].w;
+        }
     if (resid) {
         const T* xr = resid + (size_t)t * d + c4 * 4;
         acc.x = to_f32(xr[0]) + acc.x;
@@ -235,42 +257,61 @@ __global__ void __launch_bounds__(256) k_combine(const float* __restrict__ yslot
     o[3] = from_f32<T>(acc.w);
 }
 
+// Tokens per weight pass: 16 while two blocks' staged rows of either kernel fit an SM, else 8.
 template <typename T>
-cudaError_t run(const ace_layer* L, const void* x, void* out, int T_, cudaStream_t s, cudaEvent_t* ev) {
+bool wide_chunk(const ace_layer_desc& D) {
+    constexpr size_t kMost = 100 << 10;
+    return 16 * (size_t)D.hidden * sizeof(T) <= kMost && 16 * (size_t)D.ffn * sizeof(float) <= kMost;
+}
+
+template <typename T, int kTC>
+cudaError_t run_chunk(const ace_layer* L, const void* x, void* out, int T_, cudaStream_t s, cudaEvent_t* ev) {
     const T* resid = L->desc.add_residual ? static_cast<const T*>(x) : nullptr;
     const ace_layer_desc& D = L->desc;
     const Workspace& W = L->ws;
     const int d = D.hidden, m = D.ffn, k = D.top_k;
-    const int grid = L->num_sms * 2;
-    const size_t smem1 = (size_t)kTC * d * sizeof(T);
-    const size_t smem2 = (size_t)kTC * m * sizeof(float);
-    k_gemv_gateup<T><<<grid, 256, smem1, s>>>((const T*)W.h, (const T*)L->w_gate, (const T*)L->w_up,
-                                              W.offsets, W.dlist, W.perm, W.meta, W.act, d, m, k);
+    const dim3 grid(L->num_sms * 2);
+    cudaError_t e = launch_pdl(k_gemv_gateup<T, kTC>, grid, dim3(256), (size_t)kTC * d * sizeof(T), s, (const T*)W.h,
+                               (const T*)L->w_gate, (const T*)L->w_up, (const int32_t*)W.offsets,
+                               (const int32_t*)W.dlist, (const int32_t*)W.perm, (const int32_t*)W.meta, W.act, d, m, k);
+    if (e != cudaSuccess) return e;
     if (ev) ace::record_stage(ev[1], s);
-    k_gemv_down<T><<<grid, 256, smem2, s>>>(W.act, (const T*)L->w_down, W.ghat, W.offsets, W.dlist, W.perm,
-                                            W.meta, W.yslot, d, m);
+    e = launch_pdl(k_gemv_down<T, kTC>, grid, dim3(256), (size_t)kTC * m * sizeof(float), s, (const float*)W.act,
+                   (const T*)L->w_down, (const float*)W.ghat, (const int32_t*)W.offsets, (const int32_t*)W.dlist,
+                   (const int32_t*)W.perm, (const int32_t*)W.meta, W.yslot, d, m);
+    if (e != cudaSuccess) return e;
     const long long n = (long long)T_ * (d / 4);
     if (ev) ace::record_stage(ev[2], s);
-    k_combine<T><<<(int)((n + 255) / 256), 256, 0, s>>>(W.yslot, W.slot_pos, resid, (T*)out, T_, d, k);
+    const dim3 cgrid((unsigned)((n + 255) / 256));
+    e = k <= 8 ? launch_pdl(k_combine<T, 8>, cgrid, dim3(256), 0, s, (const float*)W.yslot, (const int32_t*)W.slot_pos,
+                            resid, (T*)out, T_, d, k)
+               : launch_pdl(k_combine<T, kMaxTopK>, cgrid, dim3(256), 0, s, (const float*)W.yslot,
+                            (const int32_t*)W.slot_pos, resid, (T*)out, T_, d, k);
     if (ev) ace::record_stage(ev[3], s);
-    return cudaGetLastError();
+    return e;
+}
+
+template <typename T>
+cudaError_t run(const ace_layer* L, const void* x, void* out, int T_, cudaStream_t s, cudaEvent_t* ev) {
+    return wide_chunk<T>(L->desc) ? run_chunk<T, 16>(L, x, out, T_, s, ev) : run_chunk<T, 8>(L, x, out, T_, s, ev);
+}
+
+template <typename T>
+cudaError_t init(const ace_layer_desc& D) {
+    const int d = D.hidden, m = D.ffn;
+    cudaError_t e;
+    if (wide_chunk<T>(D)) {
+        e = raise_smem_limit(k_gemv_gateup<T, 16>, (int)(16 * d * sizeof(T)));
+        return e != cudaSuccess ? e : raise_smem_limit(k_gemv_down<T, 16>, (int)(16 * m * sizeof(float)));
+    }
+    e = raise_smem_limit(k_gemv_gateup<T, 8>, (int)(8 * d * sizeof(T)));
+    return e != cudaSuccess ? e : raise_smem_limit(k_gemv_down<T, 8>, (int)(8 * m * sizeof(float)));
 }
 
 }  // namespace
 
 cudaError_t gemv_init(const ace_layer* L) {
-    const int d = L->desc.hidden, m = L->desc.ffn;
-    cudaError_t e;
-    if (L->desc.dtype == ACE_BF16) {
-        e = raise_smem_limit(k_gemv_gateup<__nv_bfloat16>, (int)(kTC * d * sizeof(__nv_bfloat16)));
-        if (e != cudaSuccess) return e;
-        e = raise_smem_limit(k_gemv_down<__nv_bfloat16>, (int)(kTC * m * sizeof(float)));
-    } else {
-        e = raise_smem_limit(k_gemv_gateup<float>, (int)(kTC * d * sizeof(float)));
-        if (e != cudaSuccess) return e;
-        e = raise_smem_limit(k_gemv_down<float>, (int)(kTC * m * sizeof(float)));
-    }
-    return e;
+    return L->desc.dtype == ACE_BF16 ? init<__nv_bfloat16>(L->desc) : init<float>(L->desc);
 }
 
 cudaError_t launch_experts_gemv(const ace_layer* L, const void* x, void* out, int T, cudaStream_t s, cudaEvent_t* ev) {

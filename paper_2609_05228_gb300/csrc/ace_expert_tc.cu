@@ -326,7 +326,8 @@ __device__ __forceinline__ int ring_take_warp(const TileRing& r, RingCursor& c, 
 
 // ---------------------------------------------------------------- kernel
 
-// A (M = 128) = token rows, B (N = 256) = weight rows.
+// A (M = 128) = token rows, B (N = WT) = weight rows: 256, or 128 for the router
+// of at most 128 experts.
 // EPI 0: SwiGLU into act (bf16); EPI 1: g_hat-scaled down-projection rows
 // per slot, bf16; EPI 2: router logits (fp32, + bias, / temperature).
 // EPI 0 and 1 draw their tiles from p.tile_next, in the order of the tile
@@ -337,10 +338,10 @@ __device__ __forceinline__ int ring_take_warp(const TileRing& r, RingCursor& c, 
 // stream HBM. Drawn and interleaved tiles with the L2 hints took the gate/up
 // and down GEMMs of 8192 Zipf-routed tokens on the large layer from 2.40 to
 // 2.28 ms and 4096 tokens on the d = 2048 layer from 256 to 246 us.
-template <int EPI, int STAGES>
+template <int EPI, int STAGES, int WT = 256>
 struct TcCfg {
     static constexpr int TOKTILE = 128;
-    static constexpr int WTILE = 256;
+    static constexpr int WTILE = WT;
     static constexpr int A_BYTES = TOKTILE * kBK * 2;
     static constexpr int B_BYTES = WTILE * kBK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -370,9 +371,10 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int EPI, int STAGES>
-__global__ void __launch_bounds__(TcCfg<EPI, STAGES>::THREADS, 1) k_expert_tc(const __grid_constant__ TcParams p) {
-    using C = TcCfg<EPI, STAGES>;
+template <int EPI, int STAGES, int WT = 256>
+__global__ void __launch_bounds__(TcCfg<EPI, STAGES, WT>::THREADS, 1) k_expert_tc(const __grid_constant__ TcParams p) {
+    static_assert(EPI == 2 || WT == 256, "expert GEMMs take 256 weight rows per tile");
+    using C = TcCfg<EPI, STAGES, WT>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE_BYTES);
@@ -1414,20 +1416,24 @@ cudaError_t launch_pair(const ace_layer* L, const TcParams& p, cudaStream_t s) {
 }
 
 constexpr int kStagesWide = 4;
+constexpr int kStagesNarrow = 6;      // 128-column tiles (router of at most 128 experts): 32 KB a stage
 
-template <int EPI>
+template <int EPI, int STAGES, int WT>
 cudaError_t set_attr() {
-    cudaError_t e = cudaFuncSetAttribute(k_expert_tc<EPI, kStagesWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         TcCfg<EPI, kStagesWide>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_expert_tc<EPI, STAGES, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         TcCfg<EPI, STAGES, WT>::SMEM);
     if (e != cudaSuccess) return e;
-    return prefer_shared(k_expert_tc<EPI, kStagesWide>);
+    return prefer_shared(k_expert_tc<EPI, STAGES, WT>);
 }
 
-template <int EPI>
+template <int EPI, int STAGES = kStagesWide, int WT = 256>
 cudaError_t launch_gemm(const ace_layer* L, const TcParams& p, cudaStream_t s) {
-    return launch_pdl(k_expert_tc<EPI, kStagesWide>, dim3(L->num_sms), dim3(TcCfg<EPI, kStagesWide>::THREADS),
-                      TcCfg<EPI, kStagesWide>::SMEM, s, p);
+    return launch_pdl(k_expert_tc<EPI, STAGES, WT>, dim3(L->num_sms), dim3(TcCfg<EPI, STAGES, WT>::THREADS),
+                      TcCfg<EPI, STAGES, WT>::SMEM, s, p);
 }
+
+// Experts per router tile: one 128-column tile covers up to 128 experts.
+int router_tile(const ace_layer* L) { return L->desc.n_experts <= 128 ? 128 : 256; }
 
 // Expert weights as tiles in HBM: block (e, t, kb) holds weight rows
 // [128 t, 128 t + 128) x columns [64 kb, 64 kb + 64) of expert e, 16 KB,
@@ -1517,9 +1523,10 @@ cudaError_t tc_init(ace_layer* L) {
     if (!tc_supported(L)) return cudaSuccess;
     const ace_layer_desc& D = L->desc;
     cudaError_t e;
-    if ((e = set_attr<0>()) != cudaSuccess) return e;
-    if ((e = set_attr<1>()) != cudaSuccess) return e;
-    if ((e = set_attr<2>()) != cudaSuccess) return e;
+    if ((e = set_attr<0, kStagesWide, 256>()) != cudaSuccess) return e;
+    if ((e = set_attr<1, kStagesWide, 256>()) != cudaSuccess) return e;
+    if ((e = set_attr<2, kStagesWide, 256>()) != cudaSuccess) return e;
+    if ((e = set_attr<2, kStagesNarrow, 128>()) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_expert_decode<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   DecCfg<1>::SMEM)) != cudaSuccess)
         return e;
@@ -1551,18 +1558,18 @@ cudaError_t tc_init(ace_layer* L) {
     if ((e = make_tensor_map(&L->tcm.tok2_small, L->ws.act_bf16, rows, m, 16, true)) != cudaSuccess) return e;
     if ((e = make_tensor_map(&L->tcm.tok2_big, L->ws.act_bf16, rows, m, 128, true)) != cudaSuccess) return e;
     // weight maps: W_gu [N * 2m, d] and W_down [N * d, m]
-    // router: h [Tmax, d] in 128-row boxes, W_r [N, d] in 256-row boxes
+    // router: h [Tmax, d] in 128-row boxes, W_r [N, d] in boxes of one tile's rows
     if ((e = make_tensor_map(&L->tcm.h_rows_big, L->ws.h, h_rows, d, 128, true)) != cudaSuccess) return e;
     // tiled expert weights as rows of 64 bf16 (16 KB tiles = 128 rows), copied verbatim
     if ((e = make_tensor_map(&L->tcm.wgu_rows, L->w_gu, n * 2 * m * d / 64, 64, 128, false)) != cudaSuccess) return e;
     if ((e = make_tensor_map(&L->tcm.wd_rows, L->w_down, n * d * m / 64, 64, 128, false)) != cudaSuccess) return e;
-    if ((e = make_tensor_map(&L->tcm.w_router_big, L->router_w, n_pad, d, 256, true)) != cudaSuccess) return e;
+    if ((e = make_tensor_map(&L->tcm.w_router_big, L->router_w, n_pad, d, router_tile(L), true)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
 // Router logits on the tensor cores for batches over 256 tokens (smaller
-// ones are routed by the fused kernel): 128 tokens x 256 experts per tile,
-// so W_r (N padded to 256 rows) is re-read from L2 once per 128 tokens.
+// ones are routed by the fused kernel): 128 tokens x 256 (or 128) experts per
+// tile, so W_r (padded to whole tiles) is re-read from L2 once per 128 tokens.
 int router_splits(const ace_layer* L, int T) {
     const ace_layer_desc& D = L->desc;
     const int base = ((T + 127) / 128) * ((D.n_experts + 255) / 256);
@@ -1593,7 +1600,9 @@ cudaError_t launch_router_tc(const ace_layer* L, int T, cudaStream_t s) {
     p.inv_temp = 1.0f / D.router_temp;
     p.use_temp = D.router_temp != 1.0f;
     p.n_valid_cols = D.n_experts;
-    return launch_gemm<2>(L, p, s);
+    // up to 128 experts: half the weight rows, MMAs and stage bytes of a 256-column tile (the
+    // padding rows' loads and products); the sums are the same
+    return router_tile(L) == 128 ? launch_gemm<2, kStagesNarrow, 128>(L, p, s) : launch_gemm<2>(L, p, s);
 }
 
 cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int T, ace_skip_ctl ctl, cudaStream_t s,

@@ -47,7 +47,6 @@ constexpr int kChunk = 64;            // tokens per compaction block (large-T ro
 constexpr int kTcSmallT = 256;       // tensor-core experts: decode tiling up to this many tokens
 constexpr int kMaxExperts = 1024;
 constexpr int kMaxTopK = 16;
-constexpr int kGemvTokenChunk = 8;   // tokens processed per weight pass in the GEMVs
 
 struct Workspace {
     void* h = nullptr;           // [Tmax, d] dtype: RMSNorm output
