@@ -1240,6 +1240,10 @@ __global__ void __launch_bounds__(256) k_combine_bf16(const Y* __restrict__ y, c
                                                       const __nv_bfloat16* __restrict__ resid,
                                                       __nv_bfloat16* __restrict__ out, int n_tokens, int d, int k,
                                                       int y_rows, int* __restrict__ err) {
+    // decode: the next layer's routing launches over this kernel's tail (its prologue reads
+    // layer constants only); 1 token 29.6 -> 28.4 us a call. Over the GEMMs and the other
+    // routing kernels an early launch measured slower.
+    if (sizeof(Y) == 4) pdl_trigger();
     pdl_wait();
     const int nq = d / 8;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;

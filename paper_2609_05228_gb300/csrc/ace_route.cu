@@ -80,6 +80,7 @@ __device__ __forceinline__ void cp_async16_row(uint32_t dst, const void* src) {
 template <typename T, int NV>
 __global__ void __launch_bounds__(256) k_rmsnorm(const T* __restrict__ x, const T* __restrict__ gamma,
                                                  T* __restrict__ h, int n_tokens, int d, float rms_eps) {
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char rn_rows[];      // [warps][d] staged rows
     pdl_wait();
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1063,6 +1064,7 @@ __global__ void __launch_bounds__(kChunk) k_compact_place(int n_tokens, int k, i
                                                           const int32_t* __restrict__ chunk_base,
                                                           int32_t* __restrict__ perm,
                                                           int32_t* __restrict__ slot_pos, int* err) {
+    pdl_trigger();
     constexpr int W = kChunk / 32;
     __shared__ uint32_t bm[kMaxExperts * W];
     for (int i = threadIdx.x; i < n_exp * W; i += blockDim.x) bm[i] = 0u;
