@@ -247,15 +247,14 @@ __device__ __forceinline__ float key_value(uint32_t k) {
 }
 
 template <int NPL>
-__device__ __forceinline__ void warp_topk(const float* __restrict__ zrow, int n_exp, int k, int lane,
-                                          int& my_id, float& my_z, bool& saw_nan) {
+__device__ __forceinline__ void warp_topk_regs(const float (&zv)[NPL], int n_exp, int k, int lane, int& my_id,
+                                               float& my_z, bool& saw_nan) {
     uint32_t v[NPL];
     saw_nan = false;
 #pragma unroll
     for (int j = 0; j < NPL; ++j) {
-        const int e = lane + 32 * j;
-        if (e < n_exp) {
-            float z = __ldcg(zrow + e);
+        if (lane + 32 * j < n_exp) {
+            float z = zv[j];
             if (z != z) { saw_nan = true; z = -INFINITY; }
             v[j] = order_key(z);
         } else {
@@ -309,6 +308,15 @@ __device__ __forceinline__ void warp_topk(const float* __restrict__ zrow, int n_
             if (lane == r) { my_id = (int)e; my_z = key_value(top); }
         }
     }
+}
+
+template <int NPL>
+__device__ __forceinline__ void warp_topk(const float* __restrict__ zrow, int n_exp, int k, int lane,
+                                          int& my_id, float& my_z, bool& saw_nan) {
+    float z[NPL];
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) z[j] = lane + 32 * j < n_exp ? __ldcg(zrow + lane + 32 * j) : 0.f;
+    warp_topk_regs<NPL>(z, n_exp, k, lane, my_id, my_z, saw_nan);
 }
 
 // c of a skip rule from the two views and the gate (ace_fusion).
@@ -663,36 +671,79 @@ __global__ void __launch_bounds__(kTopkWarps * 32) k_topk_score(float* __restric
                                                                 const float* __restrict__ bias, float inv_temp,
                                                                 int use_temp, int fusion) {
     __shared__ int hist[kHistBins];
+    __shared__ float s_tab[2 * kMaxExperts];     // the layer's GSP / RCR tables
     const bool ratio = mode == ACE_SKIP_RATIO;
     if (ratio)
         for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0;
+    // layer constants, read before the dependency wait
+    for (int i = threadIdx.x; i < n_exp; i += blockDim.x) {
+        s_tab[i] = __ldg(a_gsp + i);
+        s_tab[kMaxExperts + i] = __ldg(a_rcr + i);
+    }
     __syncthreads();
     pdl_wait();
     if (!ratio && blockIdx.x == 0 && threadIdx.x == 0) *tau_out = tau;
     const int t = blockIdx.x * kTopkWarps + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (t < n_tokens) {
-        if (n_split > 1) {
-            // split-K router: z = (sum of the slices in order + b) / temp
-            const size_t stride = (size_t)n_tokens * n_exp;
-            for (int e = lane; e < n_exp; e += 32) {
-                const size_t o = (size_t)t * n_exp + e;
-                float z = __ldcg(part + o);
-                for (int sp = 1; sp < n_split; ++sp) z += __ldcg(part + sp * stride + o);
-                z = z + bias[e];
-                if (use_temp) z = z * inv_temp;
-                logits[o] = z;
-            }
-            __syncwarp();
-        }
         int id;
         float zv;
         bool nan;
-        warp_topk<NPL>(logits + (size_t)t * n_exp, n_exp, k, lane, id, zv, nan);
+        const size_t row = (size_t)t * n_exp;
+        const size_t stride = (size_t)n_tokens * n_exp;      // between the slices of a split-K router:
+                                                             // z = (sum of the slices in order + b) / temp
+        if constexpr (NPL <= 8) {
+            // The lane's logits stay in registers up to the top-k. The kernel is a chain of
+            // L2 round trips, so several slices are loaded before they are added.
+            constexpr int G = NPL <= 4 ? 4 : 2;
+            float z[NPL];
+            if (n_split > 1) {
+                for (int sp = 0; sp < n_split; sp += G) {
+                    float v[G][NPL];
+#pragma unroll
+                    for (int g = 0; g < G; ++g)
+#pragma unroll
+                        for (int j = 0; j < NPL; ++j)
+                            v[g][j] = sp + g < n_split && lane + 32 * j < n_exp
+                                          ? __ldcg(part + (sp + g) * stride + row + lane + 32 * j) : 0.f;
+#pragma unroll
+                    for (int g = 0; g < G; ++g)
+#pragma unroll
+                        for (int j = 0; j < NPL; ++j)
+                            if (sp + g < n_split) z[j] = sp + g == 0 ? v[g][j] : z[j] + v[g][j];
+                }
+#pragma unroll
+                for (int j = 0; j < NPL; ++j) {
+                    const int e = lane + 32 * j;
+                    if (e < n_exp) {
+                        z[j] = z[j] + __ldg(bias + e);
+                        if (use_temp) z[j] = z[j] * inv_temp;
+                        logits[row + e] = z[j];
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < NPL; ++j) z[j] = lane + 32 * j < n_exp ? __ldcg(logits + row + lane + 32 * j) : 0.f;
+            }
+            warp_topk_regs<NPL>(z, n_exp, k, lane, id, zv, nan);
+        } else {
+            // more than 256 experts: the registers hold the keys only
+            if (n_split > 1) {
+                for (int e = lane; e < n_exp; e += 32) {
+                    float z = __ldcg(part + row + e);
+                    for (int sp = 1; sp < n_split; ++sp) z += __ldcg(part + sp * stride + row + e);
+                    z = z + bias[e];
+                    if (use_temp) z = z * inv_temp;
+                    logits[row + e] = z;
+                }
+                __syncwarp();
+            }
+            warp_topk<NPL>(logits + row, n_exp, k, lane, id, zv, nan);
+        }
         if (lane < k && !ACE_IDX_OK((unsigned)id < (unsigned)n_exp, err)) id = 0;   // tables are read at id
         const float z0 = __shfl_sync(0xffffffffu, zv, 0);
         if (__any_sync(0xffffffffu, nan) && lane == 0) atomicOr(err, kErrNumeric);
-        const SlotScore sc = score_slot(lane, k, zv, z0, lane < k ? id : 0, a_gsp, a_rcr, eps, fusion);
+        const SlotScore sc = score_slot(lane, k, zv, z0, lane < k ? id : 0, s_tab, s_tab + kMaxExperts, eps, fusion);
         const size_t base = (size_t)t * k;
         if (lane < k) {
             ids[base + lane] = id;
