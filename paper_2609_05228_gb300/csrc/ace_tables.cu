@@ -18,7 +18,7 @@
 // w_down[e][j][r] (the B operand, K-major as stored). The weights are read in
 // place: repacking them into K-major tiles first took 0.53 ms of kernels and
 // most of a 1.2 GB scratch allocation's 1 ms at d = 2048, N = 128, m = 768 (a
-// call took 2.71 ms, 1.47 without).
+// call took 2.71 ms, 1.49 without, 1.25 with the RCR chain overlapped).
 //
 // RCR (Algorithm 3; Eqs. rcr_centered_router, rcr_direction_prototype,
 // rcr_raw_amplification, rcr_layer_normalization): centred router rows
@@ -294,9 +294,18 @@ __global__ void __launch_bounds__(256) k_rcr_proto(const __nv_bfloat16* __restri
 // act_e[j] = SiLU(x_e . W_gate[e, j]) * (x_e . W_up[e, j]); grid (m / 64, N),
 // each warp 8 rows j, the input row and gamma^2 in shared memory. The rows
 // pass here anyway, so the block also sums its share of ||Gamma W_gate||_F^2
-// and ||Gamma W_up||_F^2: gamma_i^2 w^2 over 8 elements in fp32, those sums in
-// fp64, lanes and warps in a fixed order; one partial per block and path in
+// and ||Gamma W_up||_F^2: gamma_i^2 w^2 over 8 elements in fp32, a lane's sums
+// of those as an unevaluated pair of floats (TwoSum, Knuth; about 46 bits: the
+// fp64 adds would take longer than the loads), a row's pair, the lanes and the
+// warps in fp64 in a fixed order; one partial per block and path in
 // norms[path][e][block].
+__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float q) {
+    const float s = __fadd_rn(hi, q);
+    const float b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(q, b)));
+    hi = s;
+}
+
 __global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x, const float* __restrict__ gamma2,
                                                     const __nv_bfloat16* __restrict__ w_gate,
                                                     const __nv_bfloat16* __restrict__ w_up, int d, int m,
@@ -317,7 +326,7 @@ __global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x,
         const int j = blockIdx.x * 64 + warp * 8 + t;
         const uint4* g = reinterpret_cast<const uint4*>(w_gate + (e * m + j) * (long long)d);
         const uint4* u = reinterpret_cast<const uint4*>(w_up + (e * m + j) * (long long)d);
-        float sg = 0.f, su = 0.f;
+        float sg = 0.f, su = 0.f, gh = 0.f, gl = 0.f, uh = 0.f, ul = 0.f;
 #pragma unroll 4
         for (int q = lane; q < cv; q += 32) {
             float fg[8], fu[8];
@@ -331,9 +340,11 @@ __global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x,
                 qg = fmaf(gs[q * 8 + k] * fg[k], fg[k], qg);
                 qu = fmaf(gs[q * 8 + k] * fu[k], fu[k], qu);
             }
-            ng += (double)qg;
-            nu += (double)qu;
+            two_sum_add(gh, gl, qg);
+            two_sum_add(uh, ul, qu);
         }
+        ng += (double)gh + (double)gl;
+        nu += (double)uh + (double)ul;
         sg = warp_sum(sg);
         su = warp_sum(su);
         if (lane == 0) act[e * m + j] = sg / (1.0f + expf(-sg)) * su;
@@ -503,6 +514,12 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
     TAB_CK(cudaFuncSetAttribute(k_gsp_frob, cudaFuncAttributeMaxDynamicSharedMemorySize, kTabSmem));
     TAB_CK(ace::raise_smem_limit(k_rcr_gateup, d * 8));
     TAB_CK(ace::raise_smem_limit(k_rcr_down, m * 4));
+    // one shared-memory split for all of them: blocks of the RCR chain fit beside the GEMM's CTAs
+    TAB_CK(ace::prefer_shared(k_gsp_frob));
+    TAB_CK(ace::prefer_shared(k_rcr_colmean));
+    TAB_CK(ace::prefer_shared(k_rcr_proto));
+    TAB_CK(ace::prefer_shared(k_rcr_gateup));
+    TAB_CK(ace::prefer_shared(k_rcr_down));
     TAB_CK(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking));
     TAB_CK(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
     TAB_CK(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
