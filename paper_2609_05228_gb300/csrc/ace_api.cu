@@ -44,7 +44,7 @@ void free_layer(ace_layer* L) {
     void* ptrs[] = {L->router_w, L->router_b, L->w_gate, L->w_up, L->w_gu, L->w_down, L->gamma, L->a_gsp,
                     L->a_rcr, L->ws.h, L->ws.logits, L->ws.ids, L->ws.gates, L->ws.cval, L->ws.keys, L->ws.skip,
                     L->ws.ghat, L->ws.tau, L->ws.chunk_counts, L->ws.offsets, L->ws.dlist, L->ws.perm,
-                    L->ws.slot_pos, L->ws.meta, L->ws.act, L->ws.yslot, L->ws.h_perm, L->ws.act_bf16, L->ws.tt_off, L->ws.tt_tab, L->ws.dec_done, L->ws.tile_cnt, L->ws.sel_hist, L->ws.sel_cand, L->ws.err, L->ws.x_stage, L->ws.out_stage};
+                    L->ws.slot_pos, L->ws.meta, L->ws.act, L->ws.yslot, L->ws.y_rows, L->ws.act_bf16, L->ws.tt_off, L->ws.tt_tab, L->ws.dec_done, L->ws.tile_cnt, L->ws.sel_hist, L->ws.sel_cand, L->ws.err, L->ws.x_stage, L->ws.out_stage};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : L->ev)
@@ -411,7 +411,7 @@ ace_status ace_layer_create(const ace_layer_desc* desc_in, const void* router_w,
     ALLOC(W.sel_hist, (4096 + 1024) * sizeof(int32_t));
     ALLOC(W.sel_cand, slots * sizeof(uint32_t));
     if (L->tc) {
-        ALLOC(W.h_perm, slots * d * E);
+        ALLOC(W.y_rows, slots * d * E);
         ALLOC(W.act_bf16, slots * m * E);
         ALLOC(W.tt_off, (n + 1) * sizeof(int32_t));
         L->tt_cap = (int)(n + slots / 16 + 1);
@@ -421,7 +421,7 @@ ace_status ace_layer_create(const ace_layer_desc* desc_in, const void* router_w,
         ALLOC(W.act, slots * m * sizeof(float));
     }
     // fp32 per-slot expert outputs: every batch on the CUDA-core path, batches
-    // of up to 256 tokens on the tensor path (larger ones write bf16 rows over h_perm)
+    // of up to 256 tokens on the tensor path (larger ones write bf16 rows to y_rows)
     const size_t yslot_rows = L->tc ? (size_t)(D.max_tokens < 256 ? D.max_tokens : 256) * k : slots;
     ALLOC(W.yslot, yslot_rows * d * sizeof(float));
     ALLOC(W.err, sizeof(int));
@@ -541,7 +541,7 @@ ace_status forward_impl(ace_layer* L, const void* x, void* out, int T, ace_skip_
     }
     L->n_stages = ev ? ace::kNumStages : 0;
     L->last_launches = (small ? 1 : (h_ready ? 1 : 2) + ace::route_launch_count(L, T, ctl)) +
-                       (L->tc ? (small ? 2 : (ace::tc_use_pair(L, T, ctl) ? 4 : 3)) : 3);
+                       (L->tc && small ? 2 : 3);
     return ACE_OK;
 }
 

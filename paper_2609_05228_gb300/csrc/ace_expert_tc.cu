@@ -19,14 +19,12 @@
 // Warp roles (192 threads): warp 0 issues TMA loads into a STAGES-deep ring,
 // warp 1 owns TMEM and issues the MMAs (one thread), warps 2..5 run the
 // epilogue from TMEM (each warp reads its 32-lane quadrant). Two accumulator
-// buffers let the epilogue of one tile overlap the MMAs of the next. GEMM 1
-// of a prefill batch on one CTA per tile and the decode kernel have four more
-// warps (320 threads) that gather their token rows from h with 16-byte
-// cp.async straight into the stage, so no permuted copy of h is written and
-// read back; the CTA-pair GEMM 1 still loads rows gathered by k_gather_rows
-// (gathering there was measured 2x slower: the partner CTA's rows need a
-// relayed arrival per stage). Every mbarrier wait is bounded; on expiry the
-// kernel sets kErrTimeout, stops issuing work and releases TMEM before
+// buffers let the epilogue of one tile overlap the MMAs of the next. Four more
+// warps (320 threads) bring GEMM 1's token rows straight from h, so no permuted
+// copy of h is written and read back: with 16-byte cp.async into the stage in
+// the decode kernel and the prefill GEMM 1 on one CTA per tile, with gather4
+// TMA boxes in the CTA-pair GEMM 1. Every mbarrier wait is bounded; on expiry
+// the kernel sets kErrTimeout, stops issuing work and releases TMEM before
 // returning.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -351,7 +349,7 @@ struct TcCfg {
     static constexpr int BAR_BYTES = 512;                     // barriers, tile ring
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /*align*/ + BAR_BYTES + STG_BYTES;
     // GEMM 1 of a prefill batch gathers its token rows itself: four more
-    // warps copy them from h with 16-byte cp.async (no h_perm round trip)
+    // warps copy them from h with 16-byte cp.async
     static constexpr bool GATHER = EPI == 0;
     static constexpr bool DRAW = EPI != 2;                    // tiles drawn from a counter
     static constexpr int TAKERS = 1 + 4 + (GATHER ? 4 : 0);   // the MMA thread, the epilogue and the gather warps
@@ -1030,8 +1028,39 @@ constexpr int kPairHalf = 128 * kBK * 2;                   // 16 KB: 128 rows x 
 constexpr int kPairStage = 2 * kPairHalf;                  // this CTA's A + B halves
 constexpr int kPairSmem = kPairStages * kPairStage + 1024 + 256 + 4 * 4096;   // + epilogue staging
 
+// GEMM 1's token rows come straight from h: four warps (6..9) of each CTA load
+// tile::gather4 boxes (four rows of 128 bytes named by their token indices,
+// completing on the leader's barrier like every other load), so no permuted
+// copy of h is written and read back: 16384 tokens, four layers: 2690 ->
+// 2540 us, gate/up itself 1220 -> 1310 us against 280 us of gather kernels.
+// One elected thread per warp issues its 8 boxes a stage: one thread for all
+// 32 cannot keep up (about 88 cycles a box against 512 cycles of MMAs), 16
+// warps of two boxes were slower too (2825 us), and cp.async copies with a
+// remote arrival per warp and stage took twice the time (5490 us). Boxes past
+// the tile's last row are left out (stale rows only reach accumulator rows that
+// the epilogue does not read), but each warp loads at least one box a stage: a
+// warp whose loads no stage waits for could fall a round behind the ring, or
+// run one ahead, and its waits on a phase's parity would be ambiguous.
 template <int EPI>
-__global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_constant__ TcParams p) {
+struct PairCfg {
+    static constexpr int GATHER_WARPS = EPI == 0 ? 4 : 0;
+    static constexpr int THREADS = kThreads + 32 * GATHER_WARPS;
+};
+constexpr int kGatherBox = 4 * kBK * 2;                    // bytes of a gather4 box
+
+// Four rows of `map` (boxes of one row), at column x, to 512 bytes of swizzled stage.
+__device__ __forceinline__ void tma_gather4_pair(void* smem_dst, const CUtensorMap* map, uint32_t bar_cluster, int x,
+                                                 int r0, int r1, int r2, int r3) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+        ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(r0), "r"(r1), "r"(r2), "r"(r3),
+          "r"(bar_cluster)
+        : "memory");
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(PairCfg<EPI>::THREADS, 1) k_expert_pair(const __grid_constant__ TcParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kPairStages * kPairStage);
@@ -1086,8 +1115,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_consta
                     unsigned char* sa = smem + stage * kPairStage;
                     unsigned char* sb = sa + kPairHalf;
                     const uint32_t bar = mapa_shared(&full[stage], 0);
-                    if (leader) mbar_expect_tx(&full[stage], 2 * kPairStage);
-                    tma_load_2d_pair(sa, &p.tm_tok, bar, kb * kBK, t.row0 + 128 * (int)rank);
+                    // GEMM 1: the gather warps of both CTAs load the tile's boxes, each warp at least one
+                    if (leader)
+                        mbar_expect_tx(&full[stage],
+                                       EPI == 0 ? 2 * kPairHalf +
+                                                      ((t.nrows + 3) / 4 + 8 - (t.nrows + 31) / 32) * kGatherBox
+                                                : 2 * kPairStage);
+                    if (EPI == 1) tma_load_2d_pair(sa, &p.tm_tok, bar, kb * kBK, t.row0 + 128 * (int)rank);
                     // weight block (e, 2 wt + rank, kb) of the tiled layout: rows of 128 B, no swizzle
                     const int blk = ((t.e * (p.w_rows / 128) + 2 * t.wt + (int)rank) * p.w_kb + kb);
                     tma_load_2d_pair(sb, &p.tm_w, bar, 0, blk * 128);
@@ -1132,6 +1166,33 @@ __global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_consta
             }
             if (!ok) *abort_flag = 1;
         }
+    } else if (warp >= kGatherWarp0) {
+        // ------------------------------------------------ token-row gather (EPI 0: warps 6..9, both CTAs)
+        if (EPI == 0 && elect_one()) {
+            constexpr int R = 32;                            // this thread's tile rows: base .. base + R - 1
+            const int base = 128 * (int)rank + R * (warp - kGatherWarp0);
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int tile = unit; tile < n_tiles && ok; tile += n_units) {
+                const Tile t = tile_at<256, 256>(p, tile, n_tiles, kblocks);
+                int tok[R];
+#pragma unroll
+                for (int i = 0; i < R; ++i) tok[i] = p.perm[t.row0 + min(base + i, t.nrows - 1)] / p.k;
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    if (!mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
+                    unsigned char* dst = smem + stage * kPairStage + base % 128 * (kBK * 2);
+                    const uint32_t bar = mapa_shared(&full[stage], 0);
+#pragma unroll
+                    for (int q = 0; q < R; q += 4)
+                        if (q == 0 || base + q < t.nrows)
+                            tma_gather4_pair(dst + q * (kBK * 2), &p.tm_tok, bar, kb * kBK, tok[q], tok[q + 1],
+                                             tok[q + 2], tok[q + 3]);
+                    if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
+                }
+            }
+            if (!ok) *abort_flag = 1;
+        }
     } else {
         // ------------------------------------------------ epilogue (warps 2..5, both CTAs)
         const int quad = warp & 3;
@@ -1168,41 +1229,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_expert_pair(const __grid_consta
 }
 
 // ---------------------------------------------------------------- helper kernels
-
-// h_perm[r] = h[perm[r] / k]: token rows in expert-grouped order for the
-// TMA tile loads of GEMM 1. One warp per row; d <= 4096 (16 vectors per lane).
-__global__ void __launch_bounds__(256) k_gather_rows(const __nv_bfloat16* __restrict__ h,
-                                                     const int32_t* __restrict__ perm,
-                                                     const int32_t* __restrict__ meta,
-                                                     __nv_bfloat16* __restrict__ h_perm,
-                                                     int d, int k, int n_slots, int* __restrict__ err) {
-    pdl_wait();
-    const int R = meta[kMetaRetained];
-    const int nvec = d / 8;
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    // h rows are read once per retained slot (k times a token at most): keep
-    // them in L2; the h_perm rows are read once, by GEMM 1's TMA: stream them
-    const uint64_t keep = l2_policy_evict_last();
-    for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < R; r += gridDim.x * wpb) {
-        const int slot = perm[r];
-        if (!ACE_IDX_OK(r < n_slots && slot >= 0 && slot < n_slots, err)) continue;
-        const int tok = slot / k;
-        const uint4* src = reinterpret_cast<const uint4*>(h + (size_t)tok * d);
-        uint4* dst = reinterpret_cast<uint4*>(h_perm + (size_t)r * d);
-        uint4 v[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = lane + 32 * i;
-            if (c < nvec) v[i] = ld_l2_keep(src + c, keep);
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = lane + 32 * i;
-            if (c < nvec) st_stream(dst + c, v[i]);
-        }
-    }
-}
 
 // out[t, c] = (x[t, c] +) sum_{i kept, rank order} y[slot_pos[t*k+i], c]
 // (Eq. ace_sparse_output; y rows already carry g_hat). One thread per 8
@@ -1385,10 +1411,10 @@ cudaError_t set_pair_attr(const void* k) {
 }
 
 // Pair clusters that fit at once (one CTA per SM, clusters of two).
-cudaError_t max_pair_clusters(const void* k, int* n) {
+cudaError_t max_pair_clusters(const void* k, int threads, int* n) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = kPairSmem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1404,7 +1430,7 @@ template <int EPI>
 cudaError_t launch_pair(const ace_layer* L, const TcParams& p, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * L->pair_clusters);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(PairCfg<EPI>::THREADS);
     cfg.dynamicSmemBytes = kPairSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -1542,10 +1568,9 @@ cudaError_t tc_init(ace_layer* L) {
     if ((e = set_pair_attr((const void*)k_expert_pair<0>)) != cudaSuccess) return e;
     if ((e = set_pair_attr((const void*)k_expert_pair<1>)) != cudaSuccess) return e;
     int c0 = 0, c1 = 0;
-    if ((e = max_pair_clusters((const void*)k_expert_pair<0>, &c0)) != cudaSuccess) return e;
-    if ((e = max_pair_clusters((const void*)k_expert_pair<1>, &c1)) != cudaSuccess) return e;
+    if ((e = max_pair_clusters((const void*)k_expert_pair<0>, PairCfg<0>::THREADS, &c0)) != cudaSuccess) return e;
+    if ((e = max_pair_clusters((const void*)k_expert_pair<1>, PairCfg<1>::THREADS, &c1)) != cudaSuccess) return e;
     L->pair_clusters = c0 < c1 ? c0 : c1;
-    if ((e = prefer_shared(k_gather_rows)) != cudaSuccess) return e;
     // the stack's combine stages k slot-row chunks per thread: k x d x 2 bytes per block
     if ((e = raise_smem_limit(k_combine_norm<8>, 8 * D.hidden * 2)) != cudaSuccess) return e;
     if ((e = raise_smem_limit(k_combine_norm<kMaxTopK>, kMaxTopK * D.hidden * 2)) != cudaSuccess) return e;
@@ -1557,8 +1582,8 @@ cudaError_t tc_init(ace_layer* L) {
     const uint64_t h_rows = D.max_tokens < 256 ? 256 : (uint64_t)D.max_tokens;
     const uint64_t n_pad = ((uint64_t)D.n_experts + 255) / 256 * 256;
     const uint64_t n = D.n_experts, d = D.hidden, m = D.ffn;
-    // token maps: h_perm (GEMM 1) and act (GEMM 2), tiles of 16 / 128 rows
-    if ((e = make_tensor_map(&L->tcm.tok1_big, L->ws.h_perm, rows, d, 128, true)) != cudaSuccess) return e;
+    // token maps: single rows of h (the CTA-pair GEMM 1's gather4 boxes), act (GEMM 2) in tiles of 16 / 128 rows
+    if ((e = make_tensor_map(&L->tcm.h_gather, L->ws.h, h_rows, d, 1, true)) != cudaSuccess) return e;
     if ((e = make_tensor_map(&L->tcm.tok2_small, L->ws.act_bf16, rows, m, 16, true)) != cudaSuccess) return e;
     if ((e = make_tensor_map(&L->tcm.tok2_big, L->ws.act_bf16, rows, m, 128, true)) != cudaSuccess) return e;
     // weight maps: W_gu [N * 2m, d] and W_down [N * d, m]
@@ -1618,14 +1643,6 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     const int d = D.hidden, m = D.ffn, k = D.top_k;
     const bool small = T <= kTcSmallT;
     cudaError_t e = cudaSuccess;
-    // token rows in expert-grouped order for the CTA-pair GEMM 1's 256-row TMA tiles;
-    // the decode kernel and the single-CTA prefill GEMM 1 gather their rows themselves
-    if (pair) {
-        e = launch_pdl(k_gather_rows, dim3(L->num_sms * 4), dim3(256), 0, s, (const __nv_bfloat16*)W.h,
-                       (const int32_t*)W.perm, (const int32_t*)W.meta, (__nv_bfloat16*)W.h_perm, d, k,
-                       T * k, W.err);
-        if (e != cudaSuccess) return e;
-    }
     if (small) {
         // both GEMMs in one persistent launch (k_expert_decode), then the combine
         if (ev) ace::record_stage(ev[0], s);
@@ -1669,7 +1686,7 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     }
     if (ev) ace::record_stage(ev[0], s);
     TcParams p1{};
-    p1.tm_tok = L->tcm.tok1_big;
+    p1.tm_tok = L->tcm.h_gather;
     p1.w_tiles_hbm = static_cast<const uint8_t*>(L->w_gu);
     p1.w_kb = d / kBK;
     p1.offsets = W.offsets;
@@ -1701,9 +1718,8 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     p2.tile_next = W.meta + kMetaTile2;
     p2.w_tiles_hbm = static_cast<const uint8_t*>(L->w_down);
     p2.w_kb = m / kBK;
-    // y per slot: bf16 rows written over h_perm, which GEMM 1 (complete before
-    // GEMM 2 reads anything) no longer needs
-    p2.out = W.h_perm;
+    // y per slot, bf16 rows
+    p2.out = W.y_rows;
     p2.K = m;
     p2.w_rows = d;
     p2.w_tiles = d / 256;
@@ -1723,11 +1739,11 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out);
     const int yr = T * k;                     // slot rows of this batch
     if (next) {
-        const __nv_bfloat16* y = static_cast<const __nv_bfloat16*>(W.h_perm);
+        const __nv_bfloat16* y = static_cast<const __nv_bfloat16*>(W.y_rows);
         e = k <= 8 ? launch_combine_norm<8>(y, sp, resid, o, next, T, d, k, yr, W.err, s)
                    : launch_combine_norm<kMaxTopK>(y, sp, resid, o, next, T, d, k, yr, W.err, s);
     } else {
-        const __nv_bfloat16* y = static_cast<const __nv_bfloat16*>(W.h_perm);
+        const __nv_bfloat16* y = static_cast<const __nv_bfloat16*>(W.y_rows);
         e = k <= 8 ? launch_pdl(k_combine_bf16<__nv_bfloat16, 8>, grid, dim3(256), 0, s, y, sp, resid, o, T, d, k, yr,
                                 W.err)
                    : launch_pdl(k_combine_bf16<__nv_bfloat16, kMaxTopK>, grid, dim3(256), 0, s, y, sp, resid, o, T, d,

@@ -66,8 +66,7 @@ struct Workspace {
     int32_t* meta = nullptr;     // [kMetaCount]
     float* act = nullptr;        // [Tmax*k, m] fp32 (CUDA-core path)
     float* yslot = nullptr;      // [Tmax*k, d] fp32: g_hat-scaled expert outputs per retained slot
-    void* h_perm = nullptr;      // [Tmax*k, d] bf16: h rows in expert-grouped order (tensor path); for
-                                 // batches over 256 tokens GEMM 2 then writes its bf16 y rows over it
+    void* y_rows = nullptr;      // [Tmax*k, d] bf16: GEMM 2's output rows of batches over 256 tokens
     void* act_bf16 = nullptr;    // [Tmax*k, m] bf16 (tensor path)
     int32_t* tt_off = nullptr;   // [N+1] token-tile prefix over distinct experts
     int32_t* dec_done = nullptr; // [tiles of tt_tab] gate/up warps finished per token tile (decode kernel)
@@ -82,7 +81,7 @@ struct Workspace {
 
 // Tensor maps of the tensor-core expert path (built once at create time).
 struct TcMaps {
-    CUtensorMap tok1_big;               // h_perm, boxes of 128 rows
+    CUtensorMap h_gather;               // h, boxes of one row (gather4 loads of the CTA-pair GEMM 1)
     CUtensorMap tok2_small, tok2_big;   // act_bf16, boxes of 16 / 128 rows
     CUtensorMap h_rows_big, w_router_big;   // router GEMM (batches over 256 tokens): 128-row / 256-row boxes
     CUtensorMap wgu_rows, wd_rows;      // tiled W_gu / W_down as 128-B rows (CTA-pair kernel), no swizzle

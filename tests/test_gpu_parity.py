@@ -244,6 +244,9 @@ def _layer(kind):
             # the widest routing the library takes: 1024 experts, top-16 (a token's
             # 16 slots in the combine, 32 logits per lane in the top-k)
             spec, seed = synth.LayerSpec(256, 1024, 16, 128, dtype="bf16"), 11
+        elif kind == "few":
+            # three experts of very different load, top-1: token tiles of every fill
+            spec, seed = synth.LayerSpec(256, 3, 1, 128, dtype="bf16", zipf=True, zipf_beta=0.8), 13
         else:
             raise KeyError(kind)
         w = synth.make_layer(spec, seed)
@@ -312,6 +315,10 @@ FORWARD_CASES = [
     ("qwen_temp", 64, "ratio", 0.5), ("qwen_temp", 600, "ratio", 0.625), ("qwen_temp", 48, "threshold", 0.1),
     ("qwen", 256, "ratio", 0.5), ("qwen", 257, "ratio", 0.5),          # both sides of the small-batch path
     ("wide", 40, "ratio", 0.5), ("wide", 700, "ratio", 0.5), ("wide", 256, "threshold", 0.05),
+    # one CTA per tile (below 256 slots an expert on average) with experts of one and of several
+    # tiles; CTA pairs from 768 tokens on, with last tiles that leave gather warps without rows
+    ("few", 300, "threshold", 0.0), ("few", 767, "threshold", 0.0), ("few", 768, "threshold", 0.0),
+    ("few", 769, "threshold", 0.0), ("few", 1100, "threshold", 0.0), ("few", 2051, "threshold", 0.0),
 ]
 
 
