@@ -2,14 +2,16 @@
 // retained slots only, as weight-streaming GEMVs, and the gate-weighted
 // combine (Eq. ace_sparse_output).
 //
-// Work items are (distinct retained expert, slice of weight rows); the
-// blocks take equal shares of the weight rows. Each item streams its weight
-// rows once per chunk of up to TC tokens routed to that expert, with 16-byte
-// non-caching loads; the tokens' activations sit in shared memory, and a
-// warp's first weights are on their way before it stages them. Small layers
-// are bound by that chain of dependent loads and by the launches (PDL), so a
-// chunk is 16 tokens where they fit (an expert's tokens in one pass instead of
-// two): 64 tokens on the (256, 16 experts, top-4, 128) fp32 layer.
+// Work items are (distinct retained expert, slice of weight rows); the blocks
+// take equal shares of the weight rows. Each item streams its weight rows once
+// per chunk of up to TC tokens routed to that expert, with 16-byte non-caching
+// loads; the tokens' activations sit in shared memory, and a warp's first
+// weights are on their way before it stages them. Small layers are bound by
+// latency: the chain of dependent loads, the launches (PDL) and the sums over
+// the warp (warp_sum_all). 64 tokens on the (256, 16 experts, top-4, 128) fp32
+// layer: 42 us a call with 8-token chunks, one warp_sum per token and row and
+// plain launches; 37.8 with 16-token chunks (an expert's tokens in one pass
+// where they fit) and dependent launches; 26.1 with the joint sums.
 //   gate/up: act[r, j] = SiLU(h_t . W_gate[e, j]) * (h_t . W_up[e, j])
 //   down:    y[r, c]   = g_hat(r) * (act[r] . W_down[e, c])
 //   combine: out[t, c] = sum over t's kept slots, in rank order, of y[r, c]
@@ -28,6 +30,32 @@ __device__ __forceinline__ float silu(float u) { return u / (1.0f + expf(-u)); }
 __device__ __forceinline__ void block_range(long long total, long long& lo, long long& hi) {
     lo = total * blockIdx.x / gridDim.x;
     hi = total * (blockIdx.x + 1) / gridDim.x;
+}
+
+// Sums NV values over the warp at once: in each step of the butterfly a lane
+// sends one half of its values and keeps the other, so 2 NV shuffles do what NV
+// warp_sums do in 5 NV. Afterwards lane l holds the sums of values
+// [l NV / 32, (l + 1) NV / 32) in v[0..] (NV >= 32), or of value l NV / 32 (NV
+// < 32). The pairs added, and so the bits, are those of warp_sum.
+template <int NV>
+__device__ __forceinline__ void warp_sum_all(float (&v)[NV], int lane) {
+    int n = NV;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < NV / 2; ++i) {
+                if (i < n) {
+                    const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        }
+    }
 }
 
 // gate/up: one warp per row pair (W_gate[e, j], W_up[e, j]); each lane issues
@@ -79,9 +107,9 @@ __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, co
             }
             __syncthreads();
             for (int j = rb + warp; j < re; j += nwarps) {
-                float ag[kTC], au[kTC];
+                float acc[2 * kTC];                      // gate sums, then up sums
 #pragma unroll
-                for (int q = 0; q < kTC; ++q) { ag[q] = 0.f; au[q] = 0.f; }
+                for (int q = 0; q < 2 * kTC; ++q) acc[q] = 0.f;
                 for (int c0 = 0; c0 < nvec; c0 += 32 * kCh) {
                     if (j != rb + warp || c0 != 0) load(j, c0);
 #pragma unroll
@@ -98,21 +126,19 @@ __global__ void __launch_bounds__(256) k_gemv_gateup(const T* __restrict__ h, co
                                 Vec16<T>::to_float(hs[q * nvec + c], fh);
 #pragma unroll
                                 for (int t = 0; t < V; ++t) {
-                                    ag[q] = fmaf(fh[t], fg[t], ag[q]);
-                                    au[q] = fmaf(fh[t], fu[t], au[q]);
+                                    acc[q] = fmaf(fh[t], fg[t], acc[q]);
+                                    acc[kTC + q] = fmaf(fh[t], fu[t], acc[kTC + q]);
                                 }
                             }
                         }
                     }
                 }
-#pragma unroll
-                for (int q = 0; q < kTC; ++q) {
-                    if (q < ntc) {
-                        const float g = warp_sum(ag[q]);
-                        const float u = warp_sum(au[q]);
-                        if (lane == 0) act[(size_t)(r0 + tc0 + q) * m + j] = silu(g) * u;
-                    }
-                }
+                // lanes below 16 hold gate sums, the others up sums of the same tokens
+                warp_sum_all(acc, lane);
+                const float u = __shfl_xor_sync(0xffffffffu, acc[0], 16);
+                const int q = (lane & 15) * kTC / 16;
+                if (lane < 16 && lane % (16 / kTC) == 0 && q < ntc)
+                    act[(size_t)(r0 + tc0 + q) * m + j] = silu(acc[0]) * u;
             }
         }
         lo += re - rb;
@@ -171,11 +197,9 @@ __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act
             if (threadIdx.x < kTC) gs[threadIdx.x] = threadIdx.x < ntc ? ghat[perm[r0 + tc0 + threadIdx.x]] : 0.f;
             __syncthreads();
             for (int c = first; c < re; c += nwarps * kRows) {
-                float acc[kRows][kTC];
+                float acc[kTC * kRows];                  // value q * kRows + r: token q, row c + r
 #pragma unroll
-                for (int r = 0; r < kRows; ++r)
-#pragma unroll
-                    for (int q = 0; q < kTC; ++q) acc[r][q] = 0.f;
+                for (int i = 0; i < kTC * kRows; ++i) acc[i] = 0.f;
                 for (int v0 = 0; v0 < nvec; v0 += 32 * kCh) {
                     if (c != first || v0 != 0) load(c, v0);
 #pragma unroll
@@ -197,21 +221,18 @@ __global__ void __launch_bounds__(256) k_gemv_down(const float* __restrict__ act
                                     float fw[V];
                                     Vec16<T>::to_float(wv[r][i], fw);
 #pragma unroll
-                                    for (int t = 0; t < V; ++t) acc[r][q] = fmaf(a[t], fw[t], acc[r][q]);
+                                    for (int t = 0; t < V; ++t) acc[q * kRows + r] = fmaf(a[t], fw[t], acc[q * kRows + r]);
                                 }
                             }
                         }
                     }
                 }
+                warp_sum_all(acc, lane);
+                constexpr int kPer = kTC * kRows / 32;   // sums per lane
 #pragma unroll
-                for (int r = 0; r < kRows; ++r) {
-#pragma unroll
-                    for (int q = 0; q < kTC; ++q) {
-                        if (q < ntc) {
-                            const float y = warp_sum(acc[r][q]);
-                            if (lane == 0 && c + r < re) yslot[(size_t)(r0 + tc0 + q) * d + c + r] = gs[q] * y;
-                        }
-                    }
+                for (int i = 0; i < kPer; ++i) {
+                    const int q = (lane * kPer + i) / kRows, r = (lane * kPer + i) % kRows;
+                    if (q < ntc && c + r < re) yslot[(size_t)(r0 + tc0 + q) * d + c + r] = gs[q] * acc[i];
                 }
             }
         }
