@@ -44,7 +44,7 @@ void free_layer(ace_layer* L) {
     void* ptrs[] = {L->router_w, L->router_b, L->w_gate, L->w_up, L->w_gu, L->w_down, L->gamma, L->a_gsp,
                     L->a_rcr, L->ws.h, L->ws.logits, L->ws.ids, L->ws.gates, L->ws.cval, L->ws.keys, L->ws.skip,
                     L->ws.ghat, L->ws.tau, L->ws.chunk_counts, L->ws.offsets, L->ws.dlist, L->ws.perm,
-                    L->ws.slot_pos, L->ws.meta, L->ws.act, L->ws.yslot, L->ws.y_rows, L->ws.act_bf16, L->ws.tt_off, L->ws.tt_tab, L->ws.dec_done, L->ws.tile_cnt, L->ws.sel_hist, L->ws.sel_cand, L->ws.err, L->ws.x_stage, L->ws.out_stage};
+                    L->ws.slot_pos, L->ws.meta, L->ws.act, L->ws.yslot, L->ws.y_rows, L->ws.act_bf16, L->ws.tt_tab, L->ws.dec_done, L->ws.tile_cnt, L->ws.sel_hist, L->ws.sel_cand, L->ws.err, L->ws.x_stage, L->ws.out_stage};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : L->ev)
@@ -413,7 +413,6 @@ ace_status ace_layer_create(const ace_layer_desc* desc_in, const void* router_w,
     if (L->tc) {
         ALLOC(W.y_rows, slots * d * E);
         ALLOC(W.act_bf16, slots * m * E);
-        ALLOC(W.tt_off, (n + 1) * sizeof(int32_t));
         L->tt_cap = (int)(n + slots / 16 + 1);
         ALLOC(W.tt_tab, (size_t)L->tt_cap * sizeof(int4));
         ALLOC(W.dec_done, (n + slots / 16 + 1) * sizeof(int32_t));

@@ -68,7 +68,6 @@ struct Workspace {
     float* yslot = nullptr;      // [Tmax*k, d] fp32: g_hat-scaled expert outputs per retained slot
     void* y_rows = nullptr;      // [Tmax*k, d] bf16: GEMM 2's output rows of batches over 256 tokens
     void* act_bf16 = nullptr;    // [Tmax*k, m] bf16 (tensor path)
-    int32_t* tt_off = nullptr;   // [N+1] token-tile prefix over distinct experts
     int32_t* dec_done = nullptr; // [tiles of tt_tab] gate/up warps finished per token tile (decode kernel)
     int4* tt_tab = nullptr;      // [N + Tmax*k/16 + 1] token tiles: (expert, first row, rows, 0)
     int32_t* tile_cnt = nullptr; // [Tmax/8 + 1] per-token-tile tickets of the fused small-T kernel

@@ -555,18 +555,28 @@ __device__ float block_select_tau_rank(const uint32_t* keys, int n, int m, Selec
     return tau;
 }
 
+// What scan_counts_block leaves in shared memory: the tile table is filled
+// from it without reading back the arrays just written to global memory (three
+// dependent round trips of the routing's last block).
+struct ScanOut {
+    int* off;     // [n_exp + 1] first row of each expert, total
+    int* dl;      // [n_exp] distinct experts, increasing
+    int* tt;      // [n_exp + 1] token tiles before each distinct expert, total
+    int* tot;     // [2] D, token tiles
+};
+
 // Exclusive scan of cnt[0..n_exp) by the whole block (called by every
 // thread; blockDim.x a multiple of 32, at most 1024): offsets[e],
 // offsets[n_exp] = total, the distinct-expert list (increasing) and the meta
-// totals; also off_s (shared) when given. With tok_tile > 0 it also writes
-// tt_off[j] = sum over distinct experts before j of ceil(count / tok_tile)
-// (the token-tile schedule of the tensor-core experts) and tt_off[D].
+// totals, in global memory and in `so`. With tok_tile > 0 so.tt[j] = sum over
+// distinct experts before j of ceil(count / tok_tile) (the token-tile schedule
+// of the tensor-core experts).
 // Each thread scans a contiguous run of experts; the three running sums are
 // combined by warp shuffles and one pass over the per-warp totals in wsum
-// (shared, 3 x 32 ints).
+// (shared, 3 x 32 ints). Ends with a block barrier.
 __device__ void scan_counts_block(const int* cnt, int n_exp, int32_t* __restrict__ offsets,
-                                  int32_t* __restrict__ dlist, int32_t* __restrict__ meta, int* off_s,
-                                  int tok_tile, int32_t* __restrict__ tt_off, int* wsum) {
+                                  int32_t* __restrict__ dlist, int32_t* __restrict__ meta, const ScanOut& so,
+                                  int tok_tile, int* wsum) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int per = (n_exp + blockDim.x - 1) / blockDim.x;
     const int e0 = min(tid * per, n_exp), e1 = min(e0 + per, n_exp);
@@ -608,18 +618,21 @@ __device__ void scan_counts_block(const int* cnt, int n_exp, int32_t* __restrict
     for (int e = e0; e < e1; ++e) {
         const int c = cnt[e];
         offsets[e] = run;
-        if (off_s) off_s[e] = run;
+        so.off[e] = run;
         run += c;
         if (c > 0) {
-            if (tok_tile > 0) tt_off[drun] = trun;
+            so.tt[drun] = trun;
             trun += (c + tt - 1) / tt;
+            so.dl[drun] = e;
             dlist[drun++] = e;
         }
     }
     if (tid == blockDim.x - 1) {       // its running sums end at the totals
         offsets[n_exp] = run;
-        if (off_s) off_s[n_exp] = run;
-        if (tok_tile > 0) tt_off[drun] = trun;
+        so.off[n_exp] = run;
+        so.tt[drun] = trun;
+        so.tot[0] = drun;
+        so.tot[1] = tok_tile > 0 ? trun : 0;
         meta[kMetaRetained] = run;
         meta[kMetaDistinct] = drun;
         meta[kMetaTokTiles] = tok_tile > 0 ? trun : 0;
@@ -627,17 +640,16 @@ __device__ void scan_counts_block(const int* cnt, int n_exp, int32_t* __restrict
     __syncthreads();                   // wsum may be reused by the caller
 }
 
-// After scan_counts_block and a block barrier: the flat token-tile table of
-// the tensor-core experts, tt_tab[tt] = (expert, first row, rows, 0).
+// After scan_counts_block: the flat token-tile table of the tensor-core
+// experts, tt_tab[tt] = (expert, first row, rows, 0).
 // tt_cap: entries allocated in tt_tab (checked by the debug build).
-__device__ void fill_tile_table(const int32_t* offsets, const int32_t* dlist, const int32_t* tt_off,
-                                const int32_t* meta, int tok_tile, int4* tt_tab, int n_exp, int tt_cap, int* err) {
+__device__ void fill_tile_table(const ScanOut& so, int tok_tile, int4* tt_tab, int n_exp, int tt_cap, int* err) {
     if (tok_tile <= 0) return;
-    const int D = meta[kMetaDistinct];
+    const int D = so.tot[0];
     for (int j = threadIdx.x; j < D; j += blockDim.x) {
-        const int e = dlist[j];
+        const int e = so.dl[j];
         if (!ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) continue;
-        const int beg = offsets[e], cnt = offsets[e + 1] - beg, base = tt_off[j];
+        const int beg = so.off[e], cnt = so.off[e + 1] - beg, base = so.tt[j];
         for (int b = 0; b * tok_tile < cnt; ++b) {
             if (!ACE_IDX_OK(base + b >= 0 && base + b < tt_cap, err)) break;
             tt_tab[base + b] = make_int4(e, beg + b * tok_tile, min(tok_tile, cnt - b * tok_tile), 0);
@@ -1027,21 +1039,20 @@ __device__ __forceinline__ int block_exscan(int v, int* wtot, int& total) {
 // element a of the first list entry ceil((a + 1) TT / nM) - 1 and element b of
 // the second entry floor(b TT / nS). The entry's last field marks the
 // single-tile experts (their weights give way first in L2).
-__device__ void fill_tile_table_mixed(const int32_t* offsets, const int32_t* dlist, const int32_t* tt_off,
-                                      const int32_t* meta, int tok_tile, int4* tt_tab, int n_exp, int tt_cap, int* err,
+__device__ void fill_tile_table_mixed(const ScanOut& so, int tok_tile, int4* tt_tab, int n_exp, int tt_cap, int* err,
                                       int* wtot) {
-    const int D = meta[kMetaDistinct], TT = meta[kMetaTokTiles];
+    const int D = so.tot[0], TT = so.tot[1];
     const int per = (D + (int)blockDim.x - 1) / (int)blockDim.x;
     const int j0 = min((int)threadIdx.x * per, D), j1 = min(j0 + per, D);
     int singles = 0;
-    for (int j = j0; j < j1; ++j) singles += tt_off[j + 1] - tt_off[j] == 1;
+    for (int j = j0; j < j1; ++j) singles += so.tt[j + 1] - so.tt[j] == 1;
     int nS;
     int sb = block_exscan(singles, wtot, nS);            // single-tile experts before this thread's
     const unsigned long long tt = TT, ns = nS, nm = TT - nS;
     for (int j = j0; j < j1; ++j) {
-        const int e = dlist[j], base = tt_off[j], n = tt_off[j + 1] - base;
+        const int e = so.dl[j], base = so.tt[j], n = so.tt[j + 1] - base;
         if (!ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) continue;
-        const int beg = offsets[e], cnt = offsets[e + 1] - beg;
+        const int beg = so.off[e], cnt = so.off[e + 1] - beg;
         for (int b = 0; b < n; ++b) {
             const int pos = n == 1 ? (int)(sb * tt / ns) : (int)(((base - sb + b + 1) * tt + nm - 1) / nm) - 1;
             if (!ACE_IDX_OK(pos >= 0 && pos < tt_cap, err)) break;
@@ -1059,11 +1070,11 @@ __global__ void __launch_bounds__(kScanThreads) k_compact_scan(int n_exp, int n_
                                                                int32_t* __restrict__ offsets,
                                                                int32_t* __restrict__ dlist,
                                                                int32_t* __restrict__ meta, int tok_tile,
-                                                               int32_t* __restrict__ tt_off, int4* __restrict__ tt_tab,
-                                                               int tt_cap, int* err) {
+                                                               int4* __restrict__ tt_tab, int tt_cap, int* err) {
     __shared__ int wtot[32];
     __shared__ int wsum[96];
     __shared__ int cnt[kMaxExperts];
+    __shared__ int off_s[kMaxExperts + 1], dl_s[kMaxExperts], tt_s[kMaxExperts + 1], tot_s[2];
     __shared__ int s_last;
     pdl_wait();
     const int tid = threadIdx.x;
@@ -1100,12 +1111,12 @@ __global__ void __launch_bounds__(kScanThreads) k_compact_scan(int n_exp, int n_
     __threadfence();
     for (int e = tid; e < n_exp; e += blockDim.x) cnt[e] = __ldcg(offsets + e);
     __syncthreads();
-    scan_counts_block(cnt, n_exp, offsets, dlist, meta, nullptr, tok_tile, tt_off, wsum);
-    __syncthreads();
+    const ScanOut so{off_s, dl_s, tt_s, tot_s};
+    scan_counts_block(cnt, n_exp, offsets, dlist, meta, so, tok_tile, wsum);
     if (tok_tile == 128)
-        fill_tile_table_mixed(offsets, dlist, tt_off, meta, tok_tile, tt_tab, n_exp, tt_cap, err, wtot);
+        fill_tile_table_mixed(so, tok_tile, tt_tab, n_exp, tt_cap, err, wtot);
     else
-        fill_tile_table(offsets, dlist, tt_off, meta, tok_tile, tt_tab, n_exp, tt_cap, err);
+        fill_tile_table(so, tok_tile, tt_tab, n_exp, tt_cap, err);
 }
 
 __global__ void __launch_bounds__(kChunk) k_compact_place(int n_tokens, int k, int n_exp, int n_chunks,
@@ -1205,7 +1216,6 @@ struct FusedArgs {
     int32_t* meta;
     int* err;
     int tok_tile;
-    int32_t* tt_off;
     int4* tt_tab;
     int tt_cap;                 // entries allocated in tt_tab
     int32_t* tile_cnt;
@@ -1216,14 +1226,14 @@ struct FusedArgs {
 
 __host__ __device__ inline size_t fused_phase_c_bytes(int T, int k, int n_exp) {
     const size_t ns = (size_t)T * k;
-    return 16 + ns * 16 + (size_t)n_exp * 4 + (size_t)(n_exp + 1) * 4 + (size_t)n_exp * 32 + ns + 16;
+    return 16 + ns * 16 + (size_t)n_exp * 4 + (size_t)(3 * n_exp + 2) * 4 + (size_t)n_exp * 32 + ns + 16;
 }
 
 template <typename T, int NPL, bool LOGITS>
 __global__ void __launch_bounds__(kFuseWarps * 32) k_route_fused(const __grid_constant__ FusedArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ SelectSmem<kFuseWarps> S;
-    __shared__ int s_last;
+    __shared__ int s_last, s_tot[2];
     __shared__ float s_tab[LOGITS ? 2 * kMaxExperts : 1];   // the layer's GSP / RCR tables (phase B)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t0 = blockIdx.x * kFuseTok;
@@ -1437,7 +1447,9 @@ __global__ void __launch_bounds__(kFuseWarps * 32) k_route_fused(const __grid_co
     int* id_s = reinterpret_cast<int*>(key_s + ns);
     int* cnt = id_s + ns;                                            // [n_exp]
     int* off_s = cnt + n_exp;                                        // [n_exp + 1]
-    uint32_t* bm = reinterpret_cast<uint32_t*>(off_s + n_exp + 1);   // [n_exp * 8]
+    int* dl_s = off_s + n_exp + 1;                                   // [n_exp]
+    int* tt_s = dl_s + n_exp;                                        // [n_exp + 1]
+    uint32_t* bm = reinterpret_cast<uint32_t*>(tt_s + n_exp + 1);    // [n_exp * 8]
     uint8_t* skip_s = reinterpret_cast<uint8_t*>(bm + n_exp * 8);    // [ns]
     // ---------------- phase B: top-k, gates, c for this token tile
     const bool ratio = a.mode == ACE_SKIP_RATIO;
@@ -1533,13 +1545,13 @@ __global__ void __launch_bounds__(kFuseWarps * 32) k_route_fused(const __grid_co
         atomicOr(&bm[e * 8 + (t >> 5)], 1u << (t & 31));
     }
     __syncthreads();
-    scan_counts_block(cnt, n_exp, a.offsets, a.dlist, a.meta, off_s, a.tok_tile, a.tt_off, S.hist);
-    __syncthreads();
+    const ScanOut so{off_s, dl_s, tt_s, s_tot};
+    scan_counts_block(cnt, n_exp, a.offsets, a.dlist, a.meta, so, a.tok_tile, S.hist);
     if (a.dec_done) {                     // the decode expert kernel counts up from zero
-        for (int i = threadIdx.x; i < a.meta[kMetaTokTiles]; i += blockDim.x) a.dec_done[i] = 0;
+        for (int i = threadIdx.x; i < s_tot[1]; i += blockDim.x) a.dec_done[i] = 0;
         if (threadIdx.x == 0) a.meta[kMetaDecNext] = 0;
     }
-    fill_tile_table(a.offsets, a.dlist, a.tt_off, a.meta, a.tok_tile, a.tt_tab, n_exp, a.tt_cap, a.err);
+    fill_tile_table(so, a.tok_tile, a.tt_tab, n_exp, a.tt_cap, a.err);
     for (int s = threadIdx.x; s < ns; s += blockDim.x) {
         if (skip_s[s]) { a.slot_pos[s] = -1; continue; }
         const int e = id_s[s], t = s / k, w = t >> 5;
@@ -1683,12 +1695,15 @@ cudaError_t launch_route_fused(const ace_layer* L, const void* x, const float* l
     a.meta = W.meta;
     a.err = W.err;
     a.tok_tile = L->tc ? tc_token_tile(L, T, ctl) : 0;
-    a.tt_off = W.tt_off;
     a.tt_tab = W.tt_tab;
     a.tt_cap = L->tt_cap;
     a.tile_cnt = W.tile_cnt;
     if (x && L->tc) a.dec_done = W.dec_done;
-    if (x && L->tc && L->w_gu) {
+    // One token tile has only n_experts / 8 blocks to issue the prefetches: they take longer
+    // than the rest of the routing and hold the kernel open, for experts that few tokens keep
+    // (1 token 28.6 us a call with, 26.4 without; 8 tokens 55.8 and 54.9; 16 tokens on the
+    // large layer 251.3 and 252.8).
+    if (x && L->tc && L->w_gu && T > kFuseTok) {
         const long long gu_bytes = 2LL * D.ffn * D.hidden * 2 * D.n_experts;
         const long long want = kRoutePrefetchBytes;
         a.pf_base = static_cast<const uint8_t*>(L->w_gu);
@@ -1773,7 +1788,7 @@ cudaError_t launch_route(const ace_layer* L, const float* logits, int T, ace_ski
                    (const float*)W.tau, D.min_active, D.eps, W.ghat, W.chunk_counts, W.err);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k_compact_scan, dim3(n), dim3(kScanThreads), 0, s, n, n_chunks, W.chunk_counts, W.offsets, W.dlist,
-                   W.meta, tok_tile, W.tt_off, W.tt_tab, L->tt_cap, W.err);
+                   W.meta, tok_tile, W.tt_tab, L->tt_cap, W.err);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_compact_place, dim3(n_chunks), dim3(kChunk), 0, s, T, k, n, n_chunks, (const int32_t*)W.ids,
                       (const uint8_t*)W.skip, (const int32_t*)W.offsets, (const int32_t*)W.chunk_counts, W.perm,
