@@ -244,6 +244,8 @@ def _layer(kind):
             # the widest routing the library takes: 1024 experts, top-16 (a token's
             # 16 slots in the combine, 32 logits per lane in the top-k)
             spec, seed = synth.LayerSpec(256, 1024, 16, 128, dtype="bf16"), 11
+        elif kind == "narrow_ffn":
+            spec, seed = synth.LayerSpec(768, 16, 4, 384, dtype="bf16"), 17
         elif kind == "few":
             # three experts of very different load, top-1: token tiles of every fill
             spec, seed = synth.LayerSpec(256, 3, 1, 128, dtype="bf16", zipf=True, zipf_beta=0.8), 13
@@ -315,6 +317,11 @@ FORWARD_CASES = [
     ("qwen_temp", 64, "ratio", 0.5), ("qwen_temp", 600, "ratio", 0.625), ("qwen_temp", 48, "threshold", 0.1),
     ("qwen", 256, "ratio", 0.5), ("qwen", 257, "ratio", 0.5),          # both sides of the small-batch path
     ("wide", 40, "ratio", 0.5), ("wide", 700, "ratio", 0.5), ("wide", 256, "threshold", 0.05),
+    # decode with 64-row weight tiles (few expected slots) and the first sizes on 128-row ones;
+    # "few" and "narrow_ffn": down projections of 2 and 6 K blocks, half a stage left over
+    ("qwen", 2, "ratio", 0.25), ("qwen", 6, "ratio", 0.5), ("qwen", 7, "ratio", 0.5),
+    ("narrow_ffn", 1, "ratio", 0.0), ("narrow_ffn", 9, "ratio", 0.5), ("few", 1, "threshold", 0.0),
+    ("few", 16, "threshold", 0.0), ("few", 17, "threshold", 0.0),
     # one CTA per tile (below 256 slots an expert on average) with experts of one and of several
     # tiles; CTA pairs from 768 tokens on, with last tiles that leave gather warps without rows
     ("few", 300, "threshold", 0.0), ("few", 767, "threshold", 0.0), ("few", 768, "threshold", 0.0),
