@@ -1544,13 +1544,21 @@ cudaError_t launch_decode(const ace_layer* L, const DecParams& q, cudaStream_t s
     return launch_pdl(k_expert_decode<KBS, ROWS>, dim3(L->num_sms), dim3(C::THREADS), C::SMEM, s, q);
 }
 
-// 64-row weight tiles while the batch's gate/up work, as 128-row tiles of every slot expected to be
-// kept, gives the SMs at most two tiles each.
+// 64-row weight tiles, by the gate/up work in rounds of 128-row tiles over the SMs (expected
+// distinct experts of the slots expected to be kept). Up to half a round, halving the tiles puts
+// twice as many SMs to work (d = 2048, 1 token: 26.3 -> 24.6 us a call; d = 1024, 32 experts, 4
+// tokens: 21.9 -> 20.9). From there to a round the halves need a second round (2 tokens: 31.7 ->
+// 32.9); then, with a K loop long enough to hide a tile's own cost, they fill the last round better
+// (4 / 6 / 8 tokens: 40.9 -> 40.6, 49.3 -> 48.3, 57.1 -> 55.7; large layer, 1 token: 50.6 -> 48.8;
+// d = 1024, 16 tokens: 34.8 -> 35.7), until HBM bounds the kernel (12 tokens: 68.7 -> 69.4).
 bool dec_half_tiles(const ace_layer* L, int T, ace_skip_ctl ctl) {
     const ace_layer_desc& D = L->desc;
     if (T > kDecWideStageTokens) return false;
     const double keep = ctl.mode == ACE_SKIP_RATIO ? 1.0 - (double)ctl.value : 1.0;
-    return (double)T * D.top_k * keep * (2 * D.ffn / 128) <= 2.0 * L->num_sms;
+    const double slots = T * (D.top_k * keep > 1.0 ? D.top_k * keep : 1.0);       // the top-1 is always kept
+    const double experts = T == 1 ? slots : D.n_experts * (1.0 - pow(1.0 - 1.0 / D.n_experts, slots));
+    const double rounds = experts * (2 * D.ffn / 128) / L->num_sms;
+    return rounds <= 0.5 || (D.hidden >= 2048 && rounds >= 0.8 && rounds <= 2.5);
 }
 
 // Experts per router tile: one 128-column tile covers up to 128 experts.
