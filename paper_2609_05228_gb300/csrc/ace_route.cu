@@ -412,10 +412,10 @@ __device__ __forceinline__ void decide_slot(int lane, int k, float g, float c, f
 // values sit in registers (loops fully unrolled over kMaxTopK), and every
 // step -- the skip test, the restore order, the rank-order sum and the
 // division -- is the one decide_slot takes, so the bits agree.
-__device__ __forceinline__ void decide_token(const float* g_in, const float* c_in, int k, float tau, int m_min,
-                                             float eps, uint8_t* skip_out, float* ghat_out,
-                                             uint8_t* skip_copy) {
-    float g[kMaxTopK], c[kMaxTopK];
+// skipped_slots: bit j set where slot j is skipped; g = the gates, zs = the kept gates' sum + eps.
+__device__ __forceinline__ unsigned skipped_slots(const float* g_in, const float* c_in, int k, float tau, int m_min,
+                                                  float eps, float (&g)[kMaxTopK], float& zs_out) {
+    float c[kMaxTopK];
     unsigned sk = 0u;
 #pragma unroll
     for (int j = 0; j < kMaxTopK; ++j) {
@@ -438,13 +438,19 @@ __device__ __forceinline__ void decide_token(const float* g_in, const float* c_i
 #pragma unroll
     for (int j = 0; j < kMaxTopK; ++j)
         if (j < k && !((sk >> j) & 1u)) zs = __fadd_rn(zs, g[j]);
-    zs = __fadd_rn(zs, eps);
+    zs_out = __fadd_rn(zs, eps);
+    return sk;
+}
+
+__device__ __forceinline__ void decide_token(const float* g_in, const float* c_in, int k, float tau, int m_min,
+                                             float eps, uint8_t* skip_out, float* ghat_out) {
+    float g[kMaxTopK], zs;
+    const unsigned sk = skipped_slots(g_in, c_in, k, tau, m_min, eps, g, zs);
 #pragma unroll
     for (int j = 0; j < kMaxTopK; ++j) {
         if (j < k) {
             const bool s = (sk >> j) & 1u;
             skip_out[j] = s ? 1 : 0;
-            if (skip_copy) skip_copy[j] = s ? 1 : 0;
             ghat_out[j] = s ? 0.f : __fdiv_rn(g[j], zs);
         }
     }
@@ -527,25 +533,32 @@ __device__ float block_select_tau(const uint32_t* keys, int n, int m, SelectSmem
 // (not protected) is v when lt_i <= m < le_i, with lt_i = #{keys < key i} and
 // le_i = #{keys <= key i} (a protected 0xffffffff key is above every
 // candidate, so it counts in neither); then lo = lt_i and hi = le_i. One pass
-// over the keys and one barrier, against the radix select's four passes of
-// five barriers each: faster up to about 128 keys. The caller sets S.prefix /
-// S.below / S.last_cnt beforehand and synchronises (the values stay if no key
+// over the keys (four a load; both counts in one register) and one barrier,
+// against the radix select's four passes of five barriers each: faster up to
+// about 128 keys (at 256 keys, 32 tokens: 123.3 us a call, 121.8 with the radix
+// select). `keys` is 16-byte aligned shared memory. The caller sets S.prefix / S.below /
+// S.last_cnt beforehand and synchronises (the values stay if no key
 // qualifies, which 0 < m < #candidates rules out).
 template <int NW>
 __device__ float block_select_tau_rank(const uint32_t* keys, int n, int m, SelectSmem<NW>& S) {
     const int i = threadIdx.x;
     const uint32_t ki = i < n ? keys[i] : 0xffffffffu;
-    int lt = 0, le = 0;
-#pragma unroll 8
-    for (int j = 0; j < n; ++j) {
-        const uint32_t kj = keys[j];
-        lt += kj < ki;
-        le += kj <= ki;
-    }
-    if (ki != 0xffffffffu && lt <= m && m < le) {
-        S.prefix = ki;
-        S.below = lt;
-        S.last_cnt = le - lt;
+    if (i - (i & 31) < n) {                      // warps that hold a key
+        uint32_t cnt = 0u;                       // lt | le << 16
+        const uint4* k4 = reinterpret_cast<const uint4*>(keys);
+#pragma unroll 4
+        for (int j = 0; j < n / 4; ++j) {
+            const uint4 k = k4[j];
+            cnt += (k.x < ki) + (k.y < ki) + (k.z < ki) + (k.w < ki);
+            cnt += ((k.x <= ki) + (k.y <= ki) + (k.z <= ki) + (k.w <= ki)) << 16;
+        }
+        for (int j = n & ~3; j < n; ++j) cnt += (keys[j] < ki) + ((keys[j] <= ki) << 16);
+        const int lt = (int)(cnt & 0xffffu), le = (int)(cnt >> 16);
+        if (ki != 0xffffffffu && lt <= m && m < le) {
+            S.prefix = ki;
+            S.below = lt;
+            S.last_cnt = le - lt;
+        }
     }
     __syncthreads();
     const uint32_t v = S.prefix;
@@ -985,7 +998,7 @@ __global__ void __launch_bounds__(kChunk) k_compact_count(int n_tokens, int k, i
     if (t < n_tokens) {
         const size_t base = (size_t)t * k;
         if (DECIDE)
-            decide_token(gates + base, cval + base, k, __ldcg(tau_dev), m_min, eps, skip + base, ghat + base, nullptr);
+            decide_token(gates + base, cval + base, k, __ldcg(tau_dev), m_min, eps, skip + base, ghat + base);
         for (int i = 0; i < k; ++i) {
             const int e = ids[base + i];
             if (!skip[base + i] && ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) atomicAdd(&cnt[e], 1);
@@ -1226,7 +1239,8 @@ struct FusedArgs {
 
 __host__ __device__ inline size_t fused_phase_c_bytes(int T, int k, int n_exp) {
     const size_t ns = (size_t)T * k;
-    return 16 + ns * 16 + (size_t)n_exp * 4 + (size_t)(3 * n_exp + 2) * 4 + (size_t)n_exp * 32 + ns + 16;
+    return 16 + ns * 16 + (size_t)n_exp * 4 + (size_t)(3 * n_exp + 2) * 4 + (size_t)n_exp * 32 +
+           (size_t)T * 8 + ns + 16;
 }
 
 template <typename T, int NPL, bool LOGITS>
@@ -1441,16 +1455,18 @@ __global__ void __launch_bounds__(kFuseWarps * 32) k_route_fused(const __grid_co
     // ticket's barrier)
     const int n_tokens = a.n_tokens;
     const int ns = n_tokens * k;
-    float* g_s = reinterpret_cast<float*>(smem_raw + 16);
+    uint32_t* key_s = reinterpret_cast<uint32_t*>(smem_raw + 16);    // 16-byte aligned
+    float* g_s = reinterpret_cast<float*>(key_s + ns);
     float* c_s = g_s + ns;
-    uint32_t* key_s = reinterpret_cast<uint32_t*>(c_s + ns);
-    int* id_s = reinterpret_cast<int*>(key_s + ns);
+    int* id_s = reinterpret_cast<int*>(c_s + ns);
     int* cnt = id_s + ns;                                            // [n_exp]
     int* off_s = cnt + n_exp;                                        // [n_exp + 1]
     int* dl_s = off_s + n_exp + 1;                                   // [n_exp]
     int* tt_s = dl_s + n_exp;                                        // [n_exp + 1]
     uint32_t* bm = reinterpret_cast<uint32_t*>(tt_s + n_exp + 1);    // [n_exp * 8]
-    uint8_t* skip_s = reinterpret_cast<uint8_t*>(bm + n_exp * 8);    // [ns]
+    float* zs_s = reinterpret_cast<float*>(bm + n_exp * 8);          // [n_tokens] kept gates' sum + eps
+    unsigned* sk_s = reinterpret_cast<unsigned*>(zs_s + n_tokens);   // [n_tokens] skipped slots
+    uint8_t* skip_s = reinterpret_cast<uint8_t*>(sk_s + n_tokens);   // [ns]
     // ---------------- phase B: top-k, gates, c for this token tile
     const bool ratio = a.mode == ACE_SKIP_RATIO;
     for (int r = warp; r < nt; r += kFuseWarps) {
@@ -1528,10 +1544,21 @@ __global__ void __launch_bounds__(kFuseWarps * 32) k_route_fused(const __grid_co
         const float tau = ns <= kRankSelectMax ? block_select_tau_rank(key_s, ns, a.m_q, S)
                                                : block_select_tau(key_s, ns, a.m_q, S);
         if (threadIdx.x == 0) *a.tau_out = tau;
+        // as decide_token, in two steps: a thread per token finds the skipped slots and the gate
+        // sum, a thread per slot divides and stores (the k divisions and stores in a row took
+        // most of the 1.4 us of this step: 1 token 25.2 -> 24.6 us a call, 64 tokens 163.5 -> 162.2)
         for (int t = threadIdx.x; t < n_tokens; t += blockDim.x) {
-            const int base = t * k;
-            decide_token(g_s + base, c_s + base, k, tau, a.m_min, a.eps, a.skip + base, a.ghat + base,
-                         skip_s + base);
+            float g[kMaxTopK], zs;
+            sk_s[t] = skipped_slots(g_s + t * k, c_s + t * k, k, tau, a.m_min, a.eps, g, zs);
+            zs_s[t] = zs;
+        }
+        __syncthreads();
+        for (int s = threadIdx.x; s < ns; s += blockDim.x) {
+            const int t = s / k;
+            const bool sk = (sk_s[t] >> (s - t * k)) & 1u;
+            skip_s[s] = sk ? 1 : 0;
+            a.skip[s] = sk ? 1 : 0;
+            a.ghat[s] = sk ? 0.f : __fdiv_rn(g_s[s], zs_s[t]);
         }
         __syncthreads();
     } else if (threadIdx.x == 0) {
