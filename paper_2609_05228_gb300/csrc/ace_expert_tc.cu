@@ -685,8 +685,9 @@ struct DecParams {
 // about 0.25 us on one SM), so a lone SM streams about twice as fast with 36 KB
 // stages as with 18 KB ones: batches that retain few experts, where few SMs
 // have work, take KBS = 2 (the two K blocks of a tile are adjacent in the tiled
-// layout: one bulk copy of 32 KB); larger ones keep KBS = 1 (8 stages), which
-// every SM streams at its share of the HBM bandwidth. The smallest, whose
+// layout: one bulk copy of 32 KB), as do the largest decode batches
+// (kDecWideStageFrom); the others keep KBS = 1 (8 stages), which every SM
+// streams at its share of the HBM bandwidth. The smallest, whose
 // 128-row tiles would leave SMs without work, halve the tiles: ROWS = 64 (M =
 // 64 MMAs), KBS = 4 copies of 8 KB a stage, so that twice as many SMs stream
 // stages of the same size.
@@ -706,8 +707,13 @@ struct DecCfg {
 };
 constexpr int kDecRing = 8;             // tile indices in flight from the producer to the other roles
 constexpr int kDecRingTakers = 1 + 4 + 4;   // the MMA thread, the epilogue and the gather warps
-// Decode batches that take 2 K blocks per stage: few distinct retained experts.
+// Decode batches that take 2 K blocks per stage: up to 16 tokens (few distinct retained experts, few
+// SMs with work), and above 96, where popular experts hold several 16-token tiles whose weights come
+// from L2 at the stages' pace (d = 2048, Zipf routing, 256 tokens: 182.0 us a call with one K block,
+// 178.3 with two; large layer, 128 tokens: 757.0 and 750.9). Between, two are no better (24 tokens
+// 104.3 and 104.7, 64 tokens 163.1 and 163.6).
 constexpr int kDecWideStageTokens = 16;
+constexpr int kDecWideStageFrom = 97;
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
     int v;
@@ -1760,8 +1766,8 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
         q.ready_spin = L->dbg_ready_spin > 0 ? L->dbg_ready_spin : kSpinCycles;
         q.ready_extra = L->dbg_ready_spin > 0 ? (1 << 30) : 0;
         e = dec_half_tiles(L, T, ctl) ? launch_decode<4, 64>(L, q, s)
-            : T <= kDecWideStageTokens ? launch_decode<2, 128>(L, q, s)
-                                       : launch_decode<1, 128>(L, q, s);
+            : T <= kDecWideStageTokens || T >= kDecWideStageFrom ? launch_decode<2, 128>(L, q, s)
+                                                                 : launch_decode<1, 128>(L, q, s);
         if (e != cudaSuccess) return e;
         if (ev) {                           // gate/up and down share one launch: the down stage reads 0
             ace::record_stage(ev[1], s);
