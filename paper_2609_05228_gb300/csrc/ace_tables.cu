@@ -33,6 +33,7 @@
 // bits on every run.
 #include <cuda.h>
 #include <math.h>
+#include <string.h>
 
 #include <string>
 
@@ -487,7 +488,7 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
     const size_t o_raw = take((size_t)N * 5 * 8);
     const size_t o_mean = take((size_t)d * 8), o_x = take((size_t)N * d * 4), o_qn = take((size_t)N * 8);
     const size_t o_act = take((size_t)N * m * 4), o_rcr = take((size_t)N * rcr_per * 8);
-    const size_t o_g2 = take((size_t)d * 4), o_out = take((size_t)2 * N * 4), o_err = take(4);
+    const size_t o_g2 = take((size_t)d * 4), o_out = take((size_t)(2 * N + 1) * 4);   // results, then the error word
     unsigned char* base = nullptr;
     e = cudaMalloc(&base, off);
     if (e != cudaSuccess) return tab_fail(ACE_ERR_OOM, "ace_offline_tables_device: scratch allocation failed");
@@ -496,8 +497,9 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
     const __nv_bfloat16* wu = static_cast<const __nv_bfloat16*>(w_up);
     const __nv_bfloat16* wd = static_cast<const __nv_bfloat16*>(w_down);
     float* g2 = reinterpret_cast<float*>(base + o_g2);
-    int* err = reinterpret_cast<int*>(base + o_err);
     float* out = reinterpret_cast<float*>(base + o_out);
+    int* err = reinterpret_cast<int*>(out + 2 * N);
+    float host[2 * kMaxExperts + 1];
     int herr = 0;
     // the RCR chain (HBM-bound) runs beside the GSP GEMM (tensor-bound) on a stream of the call
     cudaStream_t s2 = nullptr;
@@ -566,10 +568,12 @@ extern "C" ace_status ace_offline_tables_device(int d, int N, int m, const void*
     k_tables_final<<<1, 1024, 0, s>>>(reinterpret_cast<const double*>(base + o_raw),
                                       reinterpret_cast<const double*>(base + o_qn), N, eps, out, out + N);
     TAB_CK(cudaGetLastError());
-    TAB_CK(cudaMemcpyAsync(gsp_out, out, (size_t)N * 4, cudaMemcpyDeviceToHost, s));
-    TAB_CK(cudaMemcpyAsync(rcr_out, out + N, (size_t)N * 4, cudaMemcpyDeviceToHost, s));
-    TAB_CK(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s));
+    // one copy: each pageable one costs about 15 us
+    TAB_CK(cudaMemcpyAsync(host, out, (size_t)(2 * N + 1) * 4, cudaMemcpyDeviceToHost, s));
     TAB_CK(cudaStreamSynchronize(s));
+    memcpy(gsp_out, host, (size_t)N * 4);
+    memcpy(rcr_out, host + N, (size_t)N * 4);
+    memcpy(&herr, host + 2 * N, 4);
     if (herr & kErrTimeout) st = tab_fail(ACE_ERR_TIMEOUT, "ace_offline_tables_device: a bounded device wait ran out");
 #undef TAB_CK
 done:
