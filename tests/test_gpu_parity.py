@@ -326,6 +326,8 @@ FORWARD_CASES = [
     # tiles; CTA pairs from 768 tokens on, with last tiles that leave gather warps without rows
     ("few", 300, "threshold", 0.0), ("few", 767, "threshold", 0.0), ("few", 768, "threshold", 0.0),
     ("few", 769, "threshold", 0.0), ("few", 1100, "threshold", 0.0), ("few", 2051, "threshold", 0.0),
+    # the combine by a block per token (hidden 512 and up; "few" and "wide" stay on the other one)
+    ("narrow_ffn", 300, "ratio", 0.5), ("narrow_ffn", 97, "ratio", 0.25),   # 97: two K blocks a stage again
 ]
 
 
