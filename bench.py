@@ -732,7 +732,7 @@ def time_tables(torch, w, reps=3):
     flops = 2 * 2 * d * d * m * n
     return {"call_ms": round(t * 1e3, 3), "gsp_gemm_tflop": round(flops / 1e12, 4),
             "gsp_gemm_tflops_over_call": round(flops / t / 1e12, 1),
-            "note": "whole call: scratch allocation, packing, GSP GEMM, norms, RCR GEMV, normalisation"}
+            "note": "whole call: scratch allocation, GSP GEMM, norms, RCR GEMV, normalisation"}
 
 
 def cpu_baseline(ws, wl, budget_s=12.0, fusion="max"):
