@@ -408,10 +408,10 @@ __device__ __forceinline__ void decide_slot(int lane, int k, float g, float c, f
     ghat_out = (on && !skip) ? __fdiv_rn(g, zs) : 0.f;
 }
 
-// The same decision with one thread per token: the token's k gates and c
+// The same decision without a warp per token: the token's k gates and c
 // values sit in registers (loops fully unrolled over kMaxTopK), and every
 // step -- the skip test, the restore order, the rank-order sum and the
-// division -- is the one decide_slot takes, so the bits agree.
+// division (left to the caller) -- is the one decide_slot takes, so the bits agree.
 // skipped_slots: bit j set where slot j is skipped; g = the gates, zs = the kept gates' sum + eps.
 __device__ __forceinline__ unsigned skipped_slots(const float* g_in, const float* c_in, int k, float tau, int m_min,
                                                   float eps, float (&g)[kMaxTopK], float& zs_out) {
@@ -440,20 +440,6 @@ __device__ __forceinline__ unsigned skipped_slots(const float* g_in, const float
         if (j < k && !((sk >> j) & 1u)) zs = __fadd_rn(zs, g[j]);
     zs_out = __fadd_rn(zs, eps);
     return sk;
-}
-
-__device__ __forceinline__ void decide_token(const float* g_in, const float* c_in, int k, float tau, int m_min,
-                                             float eps, uint8_t* skip_out, float* ghat_out) {
-    float g[kMaxTopK], zs;
-    const unsigned sk = skipped_slots(g_in, c_in, k, tau, m_min, eps, g, zs);
-#pragma unroll
-    for (int j = 0; j < kMaxTopK; ++j) {
-        if (j < k) {
-            const bool s = (sk >> j) & 1u;
-            skip_out[j] = s ? 1 : 0;
-            ghat_out[j] = s ? 0.f : __fdiv_rn(g[j], zs);
-        }
-    }
 }
 
 // --------------------------------------------------------------------------
@@ -980,33 +966,63 @@ __global__ void __launch_bounds__(1024) k_sel_final(int m, int32_t* __restrict__
 //   counts[e][c] + rank, the rank within (chunk, expert) from a per-expert
 //   token bitmap, so the order is deterministic.
 // With DECIDE (ratio mode) pass A first takes each token's decision from the
-// stored g, c and the device tau (decide_token).
+// stored g, c and the device tau (skipped_slots, then a thread per slot for the
+// division), as decide_slot does.
+// Passes A and C are chains of a few load latencies: a block of kCompactThreads
+// takes a chunk's slots side by side, up to kSlotsPerThread a thread (777
+// tokens 235.7 -> 231.8 us a call, 4096 tokens 305.4 -> 303.4, against a thread
+// per token that walked its slots).
+constexpr int kCompactThreads = 256;
+constexpr int kSlotsPerThread = kChunk * kMaxTopK / kCompactThreads;
+
 template <bool DECIDE>
-__global__ void __launch_bounds__(kChunk) k_compact_count(int n_tokens, int k, int n_exp, int n_chunks,
-                                                          const int32_t* __restrict__ ids,
-                                                          uint8_t* __restrict__ skip,
-                                                          const float* __restrict__ gates,
-                                                          const float* __restrict__ cval,
-                                                          const float* __restrict__ tau_dev, int m_min, float eps,
-                                                          float* __restrict__ ghat,
-                                                          int32_t* __restrict__ chunk_counts, int* err) {
+__global__ void __launch_bounds__(kCompactThreads) k_compact_count(int n_tokens, int k, int n_exp, int n_chunks,
+                                                                   const int32_t* __restrict__ ids,
+                                                                   uint8_t* __restrict__ skip,
+                                                                   const float* __restrict__ gates,
+                                                                   const float* __restrict__ cval,
+                                                                   const float* __restrict__ tau_dev, int m_min,
+                                                                   float eps, float* __restrict__ ghat,
+                                                                   int32_t* __restrict__ chunk_counts, int* err) {
     __shared__ int cnt[kMaxExperts];
+    __shared__ unsigned sk_s[kChunk];
+    __shared__ float zs_s[kChunk];
     for (int e = threadIdx.x; e < n_exp; e += blockDim.x) cnt[e] = 0;
-    __syncthreads();
     pdl_wait();
-    const int t = blockIdx.x * kChunk + threadIdx.x;
-    if (t < n_tokens) {
-        const size_t base = (size_t)t * k;
-        if (DECIDE)
-            decide_token(gates + base, cval + base, k, __ldcg(tau_dev), m_min, eps, skip + base, ghat + base);
-        for (int i = 0; i < k; ++i) {
-            const int e = ids[base + i];
-            if (!skip[base + i] && ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) atomicAdd(&cnt[e], 1);
-        }
+    const int t0 = blockIdx.x * kChunk, ns = min(kChunk, n_tokens - t0) * k;
+    const size_t base = (size_t)t0 * k;
+    int e[kSlotsPerThread];
+    float g[kSlotsPerThread];
+#pragma unroll
+    for (int j = 0; j < kSlotsPerThread; ++j) {
+        const int s = threadIdx.x + j * kCompactThreads;
+        e[j] = s < ns ? ids[base + s] : -1;
+        g[j] = DECIDE && s < ns ? gates[base + s] : 0.f;
+    }
+    if (DECIDE && (int)threadIdx.x < kChunk && t0 + (int)threadIdx.x < n_tokens) {
+        float gt[kMaxTopK], zs;
+        const size_t tb = base + (size_t)threadIdx.x * k;
+        sk_s[threadIdx.x] = skipped_slots(gates + tb, cval + tb, k, __ldcg(tau_dev), m_min, eps, gt, zs);
+        zs_s[threadIdx.x] = zs;
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < n_exp; e += blockDim.x)
-        chunk_counts[(size_t)e * n_chunks + blockIdx.x] = cnt[e];
+#pragma unroll
+    for (int j = 0; j < kSlotsPerThread; ++j) {
+        const int s = threadIdx.x + j * kCompactThreads;
+        if (s >= ns) break;
+        bool sk;
+        if (DECIDE) {
+            const int t = s / k;
+            sk = (sk_s[t] >> (s - t * k)) & 1u;
+            skip[base + s] = sk ? 1 : 0;
+            ghat[base + s] = sk ? 0.f : __fdiv_rn(g[j], zs_s[t]);
+        } else {
+            sk = skip[base + s];
+        }
+        if (!sk && ACE_IDX_OK((unsigned)e[j] < (unsigned)n_exp, err)) atomicAdd(&cnt[e[j]], 1);
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < n_exp; x += blockDim.x) chunk_counts[(size_t)x * n_chunks + blockIdx.x] = cnt[x];
 }
 
 constexpr int kScanThreads = 256;   // k_compact_scan block: 4 counts per thread per round
@@ -1132,43 +1148,49 @@ __global__ void __launch_bounds__(kScanThreads) k_compact_scan(int n_exp, int n_
         fill_tile_table(so, tok_tile, tt_tab, n_exp, tt_cap, err);
 }
 
-__global__ void __launch_bounds__(kChunk) k_compact_place(int n_tokens, int k, int n_exp, int n_chunks,
-                                                          const int32_t* __restrict__ ids,
-                                                          const uint8_t* __restrict__ skip,
-                                                          const int32_t* __restrict__ offsets,
-                                                          const int32_t* __restrict__ chunk_base,
-                                                          int32_t* __restrict__ perm,
-                                                          int32_t* __restrict__ slot_pos, int* err) {
+__global__ void __launch_bounds__(kCompactThreads) k_compact_place(int n_tokens, int k, int n_exp, int n_chunks,
+                                                                   const int32_t* __restrict__ ids,
+                                                                   const uint8_t* __restrict__ skip,
+                                                                   const int32_t* __restrict__ offsets,
+                                                                   const int32_t* __restrict__ chunk_base,
+                                                                   int32_t* __restrict__ perm,
+                                                                   int32_t* __restrict__ slot_pos, int* err) {
     pdl_trigger();
     constexpr int W = kChunk / 32;
     __shared__ uint32_t bm[kMaxExperts * W];
     for (int i = threadIdx.x; i < n_exp * W; i += blockDim.x) bm[i] = 0u;
     __syncthreads();
     pdl_wait();
-    const int t = blockIdx.x * kChunk + threadIdx.x;
-    const int w = threadIdx.x >> 5;
-    const unsigned bit = 1u << (threadIdx.x & 31);
-    if (t < n_tokens) {
-        for (int i = 0; i < k; ++i) {
-            const int e = ids[(size_t)t * k + i];
-            if (!skip[(size_t)t * k + i] && ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) atomicOr(&bm[e * W + w], bit);
-        }
+    const int t0 = blockIdx.x * kChunk, ns = min(kChunk, n_tokens - t0) * k;
+    const size_t base = (size_t)t0 * k;
+    int e[kSlotsPerThread], row[kSlotsPerThread];          // expert, first row of the chunk's slots of it; -1: skipped
+#pragma unroll
+    for (int j = 0; j < kSlotsPerThread; ++j) {
+        const int s = threadIdx.x + j * kCompactThreads;
+        e[j] = s < ns && !skip[base + s] ? ids[base + s] : -1;
+        if (e[j] >= 0 && !ACE_IDX_OK((unsigned)e[j] < (unsigned)n_exp, err)) e[j] = -1;
+    }
+#pragma unroll
+    for (int j = 0; j < kSlotsPerThread; ++j) {
+        if (e[j] < 0) continue;
+        const int t = (threadIdx.x + j * kCompactThreads) / k;
+        row[j] = __ldcg(offsets + e[j]) + __ldcg(chunk_base + (size_t)e[j] * n_chunks + blockIdx.x);
+        atomicOr(&bm[e[j] * W + (t >> 5)], 1u << (t & 31));
     }
     __syncthreads();
-    if (t < n_tokens) {
-        const unsigned lt = lanemask_lt();
-        for (int i = 0; i < k; ++i) {
-            const size_t s = (size_t)t * k + i;
-            if (skip[s]) { slot_pos[s] = -1; continue; }
-            const int e = ids[s];
-            if (!ACE_IDX_OK((unsigned)e < (unsigned)n_exp, err)) { slot_pos[s] = -1; continue; }
-            int rank = __popc(bm[e * W + w] & lt);
-            for (int ww = 0; ww < w; ++ww) rank += __popc(bm[e * W + ww]);
-            const int r = __ldcg(offsets + e) + __ldcg(chunk_base + (size_t)e * n_chunks + blockIdx.x) + rank;
-            if (!ACE_IDX_OK(r >= 0 && (size_t)r < (size_t)n_tokens * k, err)) { slot_pos[s] = -1; continue; }
-            perm[r] = (int32_t)s;
-            slot_pos[s] = r;
+#pragma unroll
+    for (int j = 0; j < kSlotsPerThread; ++j) {
+        const int s = threadIdx.x + j * kCompactThreads;
+        if (s >= ns) break;
+        int r = -1;
+        if (e[j] >= 0) {
+            const int t = s / k, w = t >> 5;
+            r = row[j] + __popc(bm[e[j] * W + w] & ((1u << (t & 31)) - 1u));
+            for (int ww = 0; ww < w; ++ww) r += __popc(bm[e[j] * W + ww]);
+            if (!ACE_IDX_OK(r >= 0 && (size_t)r < (size_t)n_tokens * k, err)) r = -1;
         }
+        if (r >= 0) perm[r] = (int32_t)(base + s);
+        slot_pos[base + s] = r;
     }
 }
 
@@ -1544,7 +1566,7 @@ __global__ void __launch_bounds__(kFuseWarps * 32) k_route_fused(const __grid_co
         const float tau = ns <= kRankSelectMax ? block_select_tau_rank(key_s, ns, a.m_q, S)
                                                : block_select_tau(key_s, ns, a.m_q, S);
         if (threadIdx.x == 0) *a.tau_out = tau;
-        // as decide_token, in two steps: a thread per token finds the skipped slots and the gate
+        // in two steps: a thread per token finds the skipped slots and the gate
         // sum, a thread per slot divides and stores (the k divisions and stores in a row took
         // most of the 1.4 us of this step: 1 token 25.2 -> 24.6 us a call, 64 tokens 163.5 -> 162.2)
         for (int t = threadIdx.x; t < n_tokens; t += blockDim.x) {
@@ -1810,14 +1832,14 @@ cudaError_t launch_route(const ace_layer* L, const float* logits, int T, ace_ski
     }
     const int n_chunks = cdiv(T, kChunk);
     const bool dec = mode == ACE_SKIP_RATIO;
-    e = launch_pdl(dec ? k_compact_count<true> : k_compact_count<false>, dim3(n_chunks), dim3(kChunk), 0, s, T, k, n,
+    e = launch_pdl(dec ? k_compact_count<true> : k_compact_count<false>, dim3(n_chunks), dim3(kCompactThreads), 0, s, T, k, n,
                    n_chunks, (const int32_t*)W.ids, W.skip, (const float*)W.gates, (const float*)W.cval,
                    (const float*)W.tau, D.min_active, D.eps, W.ghat, W.chunk_counts, W.err);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k_compact_scan, dim3(n), dim3(kScanThreads), 0, s, n, n_chunks, W.chunk_counts, W.offsets, W.dlist,
                    W.meta, tok_tile, W.tt_tab, L->tt_cap, W.err);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_compact_place, dim3(n_chunks), dim3(kChunk), 0, s, T, k, n, n_chunks, (const int32_t*)W.ids,
+    return launch_pdl(k_compact_place, dim3(n_chunks), dim3(kCompactThreads), 0, s, T, k, n, n_chunks, (const int32_t*)W.ids,
                       (const uint8_t*)W.skip, (const int32_t*)W.offsets, (const int32_t*)W.chunk_counts, W.perm,
                       W.slot_pos, W.err);
 }
