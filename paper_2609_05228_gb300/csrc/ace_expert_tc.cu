@@ -2,16 +2,17 @@
 // slots only, as a persistent grouped GEMM on the 5th-generation tensor cores
 // (tcgen05.mma, accumulators in TMEM, operands staged by TMA).
 //
-// One kernel template serves both projections and both batch regimes:
+// Three kernels (k_expert_decode, k_expert_tc, k_expert_pair) compute:
 //   GEMM 1 (gate/up, K = d): act[r, j] = SiLU(h_r . W_gate[e, j]) * (h_r . W_up[e, j])
 //   GEMM 2 (down,    K = m): y[r, c]   = g_hat(r) * (act[r] . W_down[e, c])
 // where rows r are retained slots in expert-grouped order (the compaction's
 // permutation) and e is the slot's expert.
-//   * decode (SWAP): the 128-row MMA operand is a tile of weight rows and the
-//     N = 16 operand is up to 16 token rows of one expert, so each weight tile
-//     is streamed once and the MMA does the reduction the GEMV would do on
-//     the CUDA cores;
-//   * prefill: the 128-row operand is a tile of token rows, N = 256 weight rows.
+//   * decode: the M operand is a tile of 128 (or 64) weight rows and the N = 16
+//     operand is up to 16 token rows of one expert, so each weight tile is
+//     streamed once and the MMA does the reduction the GEMV would do on the
+//     CUDA cores;
+//   * prefill: the M operand is a tile of 128 token rows (256 on a CTA pair),
+//     N = 256 weight rows.
 // Gate and up rows are interleaved in blocks of 16 (W_gu packed at create
 // time), so one accumulator tile holds matching gate and up outputs and the
 // SiLU-and-product runs in the epilogue.

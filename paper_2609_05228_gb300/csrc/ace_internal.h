@@ -267,7 +267,7 @@ bool tc_use_pair(const ace_layer* L, int T, ace_skip_ctl ctl);
 cudaError_t tc_init(ace_layer* L);
 // Packs W_gate / W_up / W_down into the tiled, pre-swizzled layouts of w_gu and w_down.
 cudaError_t tc_pack_weights(ace_layer* L, const void* w_gate, const void* w_up, const void* w_down, cudaStream_t s);
-// ev (nullable): recorded after gather, after gate/up, after down, after combine.
+// ev (nullable): recorded before gate/up, after gate/up, after down, after combine.
 // next (nullable, T > 256 only): the following layer of a stack; the combine
 // then also writes that layer's RMSNorm of `out` into next->ws.h.
 cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int T, ace_skip_ctl ctl, cudaStream_t s,
