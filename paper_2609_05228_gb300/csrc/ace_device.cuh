@@ -190,6 +190,18 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
     return true;
 }
 
+// The same for a converged warp: lane 0 waits and every lane gets the result.
+// The shuffle that hands it out orders no memory accesses; the __syncwarp
+// puts the accesses of all lanes behind the phase that lane 0 observed.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, volatile int* abort_flag,
+                                               int lane) {
+    int ok = 1;
+    if (lane == 0) ok = mbar_wait_or_abort(bar, parity, err, abort_flag);
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();
+    return ok != 0;
+}
+
 // 1-D bulk copy global -> shared (16-byte aligned addresses, size a multiple
 // of 16), completing `bytes` of transaction count on `bar`.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {

@@ -553,9 +553,7 @@ __global__ void __launch_bounds__(TcCfg<EPI, STAGES, WT>::THREADS, 1) k_expert_t
                     nb[j] = in ? 16u : 0u;
                 }
                 for (int kb = 0; kb < kblocks; ++kb) {
-                    int go = 1;
-                    if (lane == 0) go = mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag);
-                    if (!__shfl_sync(0xffffffffu, go, 0)) { ok = false; break; }
+                    if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, abort_flag, lane)) { ok = false; break; }
                     const uint32_t sa = smem_u32(smem + stage * C::STAGE_BYTES) + (uint32_t)g * 128u + cx;
                     const int kx = (t.kb0 + kb) * kBK;
 #pragma unroll
@@ -582,10 +580,7 @@ __global__ void __launch_bounds__(TcCfg<EPI, STAGES, WT>::THREADS, 1) k_expert_t
             // the tile's rows and g_hat are read while its MMAs still run
             const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
             const float gh = wide_row_ghat<EPI>(p, t, quad * 32 + lane);
-            bool ok = true;
-            if (lane == 0) ok = mbar_wait_or_abort(&acc_full[acc], acc_phase, p.err, abort_flag);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * C::ACC_COLS);
             // lane = token row, columns = WTILE weight rows
@@ -968,9 +963,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
             const bool in = t.phase == 0 && r < t.nrows;
             const __nv_bfloat16* src = p.h + (size_t)(in ? p.perm[t.row0 + r] / p.k : 0) * p.d + c * 8;
             for (int kb = 0; kb < t.kblocks; kb += KBS) {
-                int go = 1;
-                if (lane == 0) go = mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag);
-                if (!__shfl_sync(0xffffffffu, go, 0)) { ok = false; break; }
+                if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, abort_flag, lane)) { ok = false; break; }
                 if (t.phase == 0) {
                     const uint32_t sb = smem_u32(smem + stage * kDecStage + kDecA) + off;
 #pragma unroll
@@ -1003,10 +996,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
             if (lane == 0) mbar_arrive(&ring_empty[ri]);
             if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
             if (tile < 0) break;
-            bool ok = true;
-            if (lane == 0) ok = mbar_wait_or_abort(&acc_full[acc], acc_phase, p.err, abort_flag);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
             tc_fence_after();
             const DecTile t = dec_tile<ROWS>(p, tile, n1);
             uint32_t r[16];
@@ -1018,10 +1008,8 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                 // them over in shared memory
                 const int pr = quad >> 1;
                 float* xch = reinterpret_cast<float*>(smem + kDecStages * kDecStage + 512) + pr * 256;
-                int go = 1;
                 if (quad & 1) {
-                    if (lane == 0) go = mbar_wait_or_abort(&xch_empty[pr], xch_phase ^ 1u, p.err, abort_flag);
-                    if (!__shfl_sync(0xffffffffu, go, 0)) break;
+                    if (!mbar_wait_warp(&xch_empty[pr], xch_phase ^ 1u, p.err, abort_flag, lane)) break;
                     if (lane < 16) {
 #pragma unroll
                         for (int c = 0; c < 16; ++c) xch[c * 16 + lane] = __uint_as_float(r[c]);
@@ -1029,8 +1017,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&xch_full[pr]);
                 } else {
-                    if (lane == 0) go = mbar_wait_or_abort(&xch_full[pr], xch_phase, p.err, abort_flag);
-                    if (!__shfl_sync(0xffffffffu, go, 0)) break;
+                    if (!mbar_wait_warp(&xch_full[pr], xch_phase, p.err, abort_flag, lane)) break;
                     if (lane < 16) {
                         const int j = (t.wt * 2 + pr) * 16 + lane;
 #pragma unroll
@@ -1281,10 +1268,7 @@ __global__ void __launch_bounds__(PairCfg<EPI>::THREADS, 1) k_expert_pair(const 
             // the tile's rows and g_hat are read while its MMAs still run
             const Tile t = tile_at<256, 256>(p, tile, n_tiles, kblocks);
             const float gh = wide_row_ghat<EPI>(p, t, row_base + lane);
-            bool ok = true;
-            if (lane == 0) ok = mbar_wait_or_abort(&acc_full[acc], acc_phase, p.err, abort_flag);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256);
             epilogue_wide<EPI>(p, t, tbase, row_base, lane, gh, stg);
