@@ -7,7 +7,7 @@
 //   GEMM 2 (down,    K = m): y[r, c]   = g_hat(r) * (act[r] . W_down[e, c])
 // where rows r are retained slots in expert-grouped order (the compaction's
 // permutation) and e is the slot's expert.
-//   * decode: the M operand is a tile of 128 (or 64) weight rows and the N = 16
+//   * decode: the M operand is a tile of 128 weight rows and the N = 16
 //     operand is up to 16 token rows of one expert, so each weight tile is
 //     streamed once and the MMA does the reduction the GEMV would do on the
 //     CUDA cores;
@@ -676,30 +676,30 @@ struct DecParams {
     int ready_extra;                    // added to that wait's target: 0, or unreachable (a test of the bound)
 };
 
-// A stage holds KBS K blocks of a ROWS-row weight tile, followed by KBS token
+// A stage holds KBS K blocks of a 128-row weight tile, followed by KBS token
 // boxes. Each stage costs a fixed producer / MMA / barrier round trip (measured
 // about 0.25 us on one SM), so a lone SM streams about twice as fast with 36 KB
 // stages as with 18 KB ones: batches that retain few experts, where few SMs
 // have work, take KBS = 2 (the two K blocks of a tile are adjacent in the tiled
 // layout: one bulk copy of 32 KB), as do the largest decode batches
 // (kDecWideStageFrom); the others keep KBS = 1 (8 stages), which every SM
-// streams at its share of the HBM bandwidth. The smallest, whose
-// 128-row tiles would leave SMs without work, halve the tiles: ROWS = 64 (M =
-// 64 MMAs), KBS = 4 copies of 8 KB a stage, so that twice as many SMs stream
-// stages of the same size.
-template <int KBS, int ROWS>
+// streams at its share of the HBM bandwidth. 64-row tiles (M = 64 MMAs, four 8 KB
+// copies a stage) for few expected slots, which put twice as many SMs to work, were
+// taken back: 1 token 25.8 and 25.7 us a call, 4 tokens 39.8 and 40.7, 8 tokens 56.0 and
+// 55.1; over 13 shapes at 1 to 16 tokens between 8% faster (2560 x 2048, 8 experts) and
+// 14% slower (1024 x 512, 128 experts), with no rule on the sizes that separated the two.
+template <int KBS>
 struct DecCfg {
     // warps 0-5 as in k_expert_tc; warps 6-9 gather the gate/up tiles' token
     // rows from h with cp.async (one 16-byte chunk of each row per thread and
     // K block) and arrive on every stage's full barrier
     static constexpr int THREADS = kThreads + 32 * 4;
-    static constexpr int STAGES = KBS == 1 ? 8 : (KBS == 2 ? 6 : 5);
-    static constexpr int A1 = ROWS * kBK * 2;                 // one K block of the weight tile
+    static constexpr int STAGES = KBS == 1 ? 8 : 6;
+    static constexpr int A1 = 128 * kBK * 2;                  // one K block of the weight tile
     static constexpr int A = KBS * A1;
     static constexpr int B1 = 16 * kBK * 2;                   // one token box (16 rows x 64 bf16)
     static constexpr int STAGE = A + KBS * B1;
-    static constexpr int XCH = ROWS == 64 ? 2 * 16 * 16 * 4 : 0;   // up rows handed to the gate rows' warps
-    static constexpr int SMEM = STAGES * STAGE + 1024 + 512 + XCH;
+    static constexpr int SMEM = STAGES * STAGE + 1024 + 512;
 };
 constexpr int kDecRing = 8;             // tile indices in flight from the producer to the other roles
 constexpr int kDecRingTakers = 1 + 4 + 4;   // the MMA thread, the epilogue and the gather warps
@@ -725,21 +725,13 @@ struct DecTile {
     int phase;    // 0 gate/up, 1 down
     int tt;       // token tile
     int e, row0, nrows;
-    int wt;       // weight tile (ROWS rows)
+    int wt;       // weight tile (128 rows)
     int kblocks;
 };
 
-// K blocks in the stage that starts at block kb: KBS, or what is left (K blocks are even: d is a
-// multiple of 256 and m of 128).
-template <int KBS>
-__device__ __forceinline__ int dec_stage_blocks(int kb, int kblocks) {
-    return KBS <= 2 ? KBS : min(KBS, kblocks - kb);
-}
-
-template <int ROWS>
 __device__ __forceinline__ DecTile dec_tile(const DecParams& p, int tile, int n1) {
     DecTile t;
-    const int wt1 = 2 * p.m / ROWS, wt2 = p.d / ROWS;
+    const int wt1 = 2 * p.m / 128, wt2 = p.d / 128;
     if (tile < n1) {
         t.phase = 0;
         t.tt = tile / wt1;
@@ -759,9 +751,10 @@ __device__ __forceinline__ DecTile dec_tile(const DecParams& p, int tile, int n1
     return t;
 }
 
-template <int KBS, int ROWS>
-__global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode(const __grid_constant__ DecParams p) {
-    using C = DecCfg<KBS, ROWS>;
+// K blocks come in whole stages: their count is even (d is a multiple of 256, m of 128).
+template <int KBS>
+__global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const __grid_constant__ DecParams p) {
+    using C = DecCfg<KBS>;
     constexpr int kDecStages = C::STAGES, kDecStage = C::STAGE, kDecA = C::A;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -774,9 +767,6 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_empty + kDecRing);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* ring = abort_flag + 1;        // [kDecRing] tile indices, -1 = no more
-    // 64-row tiles: an epilogue warp pair's hand-over of up rows (8-byte aligned: kDecRing is even)
-    uint64_t* xch_full = reinterpret_cast<uint64_t*>(tmem_slot + 2 + kDecRing);
-    uint64_t* xch_empty = xch_full + 2;
     const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tm_act)) : "memory");
@@ -792,10 +782,6 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
             mbar_init(&ring_full[r], 1);
             mbar_init(&ring_empty[r], kDecRingTakers);
         }
-        for (int x = 0; x < 2; ++x) {
-            mbar_init(&xch_full[x], 1);
-            mbar_init(&xch_empty[x], 1);
-        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -810,8 +796,8 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
     const uint32_t tmem_base = *tmem_slot;
     pdl_wait();
     const int ntt = p.meta[kMetaTokTiles];
-    const int wt1 = 2 * p.m / ROWS;
-    const int n1 = ntt * wt1, n_tiles = n1 + ntt * (p.d / ROWS);
+    const int wt1 = 2 * p.m / 128;
+    const int n1 = ntt * wt1, n_tiles = n1 + ntt * (p.d / 128);
     const int done_target = 4 * wt1 + p.ready_extra;
 
     if (warp == 0) {
@@ -831,7 +817,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                 mbar_arrive(&ring_full[ri]);
                 if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
                 if (tile >= n_tiles) break;
-                const DecTile t = dec_tile<ROWS>(p, tile, n1);
+                const DecTile t = dec_tile(p, tile, n1);
                 if (t.phase == 1) {
                     // the token tile's act rows: every gate/up epilogue warp has written
                     if (ld_acquire(p.done + t.tt) < done_target) {
@@ -849,27 +835,17 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                 }
                 const uint8_t* wbase = t.phase == 0 ? p.w_gu : p.w_down;
                 const int wrows = t.phase == 0 ? 2 * p.m : p.d;
-                // the tile's first K block (a 64-row tile is half of a 16 KB block)
-                const uint8_t* w0 = wbase + ((size_t)t.e * (wrows / 128) + t.wt * ROWS / 128) * t.kblocks * 16384 +
-                                    t.wt % (128 / ROWS) * C::A1;
+                const uint8_t* w0 = wbase + ((size_t)t.e * (wrows / 128) + t.wt) * t.kblocks * 16384;
                 for (int kb = 0; kb < t.kblocks; kb += KBS) {
                     if (!mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                     unsigned char* sa = smem + stage * kDecStage;
-                    const int nk = dec_stage_blocks<KBS>(kb, t.kblocks);
                     // gate/up: the gather warps copy the token rows (their own arrivals)
-                    mbar_expect_tx(&full[stage], nk * (t.phase == 0 ? C::A1 : C::A1 + C::B1));
-                    if (ROWS == 128) {
-                        bulk_g2s(sa, w0 + (size_t)kb * 16384, KBS * 16384, &full[stage]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < KBS; ++j)
-                            if (j < nk) bulk_g2s(sa + j * C::A1, w0 + (size_t)(kb + j) * 16384, C::A1, &full[stage]);
-                    }
+                    mbar_expect_tx(&full[stage], t.phase == 0 ? kDecA : kDecStage);
+                    bulk_g2s(sa, w0 + (size_t)kb * 16384, kDecA, &full[stage]);
                     if (t.phase == 1) {
 #pragma unroll
                         for (int j = 0; j < KBS; ++j)
-                            if (j < nk)
-                                tma_load_2d(sa + kDecA + j * C::B1, &p.tm_act, &full[stage], (kb + j) * kBK, t.row0);
+                            tma_load_2d(sa + kDecA + j * C::B1, &p.tm_act, &full[stage], (kb + j) * kBK, t.row0);
                     }
                     ++issued;
                     if (++stage == kDecStages) { stage = 0; phase ^= 1u; }
@@ -888,7 +864,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(ROWS, 16);
+            constexpr uint32_t idesc = idesc_bf16(128, 16);
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -902,7 +878,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                 mbar_arrive(&ring_empty[ri]);
                 if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
                 if (tile < 0) break;
-                const DecTile t = dec_tile<ROWS>(p, tile, n1);
+                const DecTile t = dec_tile(p, tile, n1);
                 if (!mbar_wait_or_abort(&acc_empty[acc], acc_phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 16);
@@ -912,10 +888,8 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     tc_fence_after();
                     const uint32_t s_addr = smem_u32(smem + stage * kDecStage);
-                    const int nk = dec_stage_blocks<KBS>(kb, t.kblocks);
 #pragma unroll
                     for (int j = 0; j < KBS; ++j) {
-                        if (j >= nk) break;
                         const uint32_t a_addr = s_addr + j * C::A1;               // weight tile kb + j
                         const uint32_t b_addr = s_addr + kDecA + j * C::B1;       // its token box
                         const uint64_t ad = smem_desc_sw128(a_addr), bd = smem_desc_sw128(b_addr);
@@ -959,7 +933,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
             if (lane == 0) mbar_arrive(&ring_empty[ri]);
             if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
             if (tile < 0) break;
-            const DecTile t = dec_tile<ROWS>(p, tile, n1);
+            const DecTile t = dec_tile(p, tile, n1);
             const bool in = t.phase == 0 && r < t.nrows;
             const __nv_bfloat16* src = p.h + (size_t)(in ? p.perm[t.row0 + r] / p.k : 0) * p.d + c * 8;
             for (int kb = 0; kb < t.kblocks; kb += KBS) {
@@ -968,7 +942,7 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                     const uint32_t sb = smem_u32(smem + stage * kDecStage + kDecA) + off;
 #pragma unroll
                     for (int j = 0; j < KBS; ++j)
-                        if (kb + j < t.kblocks) cp_async16(sb + j * C::B1, src + (kb + j) * kBK, in ? 16u : 0u);
+                        cp_async16(sb + j * C::B1, src + (kb + j) * kBK, in ? 16u : 0u);
                 }
                 cp_async_arrive_noinc(&full[stage]);
                 if (++stage == kDecStages) { stage = 0; phase ^= 1u; }
@@ -983,7 +957,6 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
         uint32_t acc_phase = 0;
         int ri = 0;
         uint32_t rph = 0;
-        uint32_t xch_phase = 0;
         while (true) {
             int tile = -1, go = 1;
             if (lane == 0) {
@@ -998,43 +971,11 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
             if (tile < 0) break;
             if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
             tc_fence_after();
-            const DecTile t = dec_tile<ROWS>(p, tile, n1);
+            const DecTile t = dec_tile(p, tile, n1);
             uint32_t r[16];
             tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 16), r);
             tmem_ld_wait();
-            if (ROWS == 64 && t.phase == 0) {
-                // M = 64: this warp's rows sit in its first 16 lanes, gate rows of FFN block
-                // 2 * wt + quad / 2 for an even quad, its up rows for the odd one, which hands
-                // them over in shared memory
-                const int pr = quad >> 1;
-                float* xch = reinterpret_cast<float*>(smem + kDecStages * kDecStage + 512) + pr * 256;
-                if (quad & 1) {
-                    if (!mbar_wait_warp(&xch_empty[pr], xch_phase ^ 1u, p.err, abort_flag, lane)) break;
-                    if (lane < 16) {
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) xch[c * 16 + lane] = __uint_as_float(r[c]);
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&xch_full[pr]);
-                } else {
-                    if (!mbar_wait_warp(&xch_full[pr], xch_phase, p.err, abort_flag, lane)) break;
-                    if (lane < 16) {
-                        const int j = (t.wt * 2 + pr) * 16 + lane;
-#pragma unroll
-                        for (int c = 0; c < 16; ++c)
-                            if (c < t.nrows)
-                                p.act[(size_t)(t.row0 + c) * p.m + j] =
-                                    __float2bfloat16_rn(silu(__uint_as_float(r[c])) * xch[c * 16 + lane]);
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&xch_empty[pr]);
-                    fence_proxy_async_global();      // act is read by the TMA of down tiles
-                    __threadfence();
-                    __syncwarp();
-                }
-                xch_phase ^= 1u;
-                if (lane == 0) atomicAdd(p.done + t.tt, 1);
-            } else if (t.phase == 0) {
+            if (t.phase == 0) {
                 // rows: 16 gate then 16 up of FFN block (4 * wt + quad); SwiGLU into act
                 const int j = (t.wt * 4 + quad) * 16 + (lane & 15);
 #pragma unroll
@@ -1049,11 +990,10 @@ __global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode
                 __syncwarp();
                 if (lane == 0) atomicAdd(p.done + t.tt, 1);
             } else {
-                // a warp's rows: 32 lanes (M = 128) or the first 16 (M = 64)
-                const int col = t.wt * ROWS + quad * (ROWS / 4) + lane;
+                const int col = t.wt * 128 + quad * 32 + lane;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
-                    if (lane < ROWS / 4 && c < t.nrows)
+                    if (c < t.nrows)
                         p.y[(size_t)(t.row0 + c) * p.d + col] = p.ghat[p.perm[t.row0 + c]] * __uint_as_float(r[c]);
                 }
             }
@@ -1535,34 +1475,17 @@ cudaError_t set_combine_attr(int d) {
     return e != cudaSuccess ? e : prefer_shared(k_combine_norm<KMAX, NORM>);
 }
 
-template <int KBS, int ROWS>
+template <int KBS>
 cudaError_t set_decode_attr() {
-    cudaError_t e = cudaFuncSetAttribute(k_expert_decode<KBS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         DecCfg<KBS, ROWS>::SMEM);
-    return e != cudaSuccess ? e : prefer_shared(k_expert_decode<KBS, ROWS>);
+    cudaError_t e = cudaFuncSetAttribute(k_expert_decode<KBS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         DecCfg<KBS>::SMEM);
+    return e != cudaSuccess ? e : prefer_shared(k_expert_decode<KBS>);
 }
 
-template <int KBS, int ROWS>
+template <int KBS>
 cudaError_t launch_decode(const ace_layer* L, const DecParams& q, cudaStream_t s) {
-    using C = DecCfg<KBS, ROWS>;
-    return launch_pdl(k_expert_decode<KBS, ROWS>, dim3(L->num_sms), dim3(C::THREADS), C::SMEM, s, q);
-}
-
-// 64-row weight tiles, by the gate/up work in rounds of 128-row tiles over the SMs (expected
-// distinct experts of the slots expected to be kept). Up to half a round, halving the tiles puts
-// twice as many SMs to work (d = 2048, 1 token: 26.3 -> 24.6 us a call; d = 1024, 32 experts, 4
-// tokens: 21.9 -> 20.9). From there to a round the halves need a second round (2 tokens: 31.7 ->
-// 32.9); then, with a K loop long enough to hide a tile's own cost, they fill the last round better
-// (4 / 6 / 8 tokens: 40.9 -> 40.6, 49.3 -> 48.3, 57.1 -> 55.7; large layer, 1 token: 50.6 -> 48.8;
-// d = 1024, 16 tokens: 34.8 -> 35.7), until HBM bounds the kernel (12 tokens: 68.7 -> 69.4).
-bool dec_half_tiles(const ace_layer* L, int T, ace_skip_ctl ctl) {
-    const ace_layer_desc& D = L->desc;
-    if (T > kDecWideStageTokens) return false;
-    const double keep = ctl.mode == ACE_SKIP_RATIO ? 1.0 - (double)ctl.value : 1.0;
-    const double slots = T * (D.top_k * keep > 1.0 ? D.top_k * keep : 1.0);       // the top-1 is always kept
-    const double experts = T == 1 ? slots : D.n_experts * (1.0 - pow(1.0 - 1.0 / D.n_experts, slots));
-    const double rounds = experts * (2 * D.ffn / 128) / L->num_sms;
-    return rounds <= 0.5 || (D.hidden >= 2048 && rounds >= 0.8 && rounds <= 2.5);
+    using C = DecCfg<KBS>;
+    return launch_pdl(k_expert_decode<KBS>, dim3(L->num_sms), dim3(C::THREADS), C::SMEM, s, q);
 }
 
 // Experts per router tile: one 128-column tile covers up to 128 experts.
@@ -1660,9 +1583,8 @@ cudaError_t tc_init(ace_layer* L) {
     if ((e = set_attr<1, kStagesWide, 256>()) != cudaSuccess) return e;
     if ((e = set_attr<2, kStagesWide, 256>()) != cudaSuccess) return e;
     if ((e = set_attr<2, kStagesNarrow, 128>()) != cudaSuccess) return e;
-    if ((e = set_decode_attr<1, 128>()) != cudaSuccess) return e;
-    if ((e = set_decode_attr<2, 128>()) != cudaSuccess) return e;
-    if ((e = set_decode_attr<4, 64>()) != cudaSuccess) return e;
+    if ((e = set_decode_attr<1>()) != cudaSuccess) return e;
+    if ((e = set_decode_attr<2>()) != cudaSuccess) return e;
     if ((e = set_pair_attr((const void*)k_expert_pair<0>)) != cudaSuccess) return e;
     if ((e = set_pair_attr((const void*)k_expert_pair<1>)) != cudaSuccess) return e;
     int c0 = 0, c1 = 0;
@@ -1763,9 +1685,7 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
         q.k = k;
         q.ready_spin = L->dbg_ready_spin > 0 ? L->dbg_ready_spin : kSpinCycles;
         q.ready_extra = L->dbg_ready_spin > 0 ? (1 << 30) : 0;
-        e = dec_half_tiles(L, T, ctl) ? launch_decode<4, 64>(L, q, s)
-            : T <= kDecWideStageTokens || T >= kDecWideStageFrom ? launch_decode<2, 128>(L, q, s)
-                                                                 : launch_decode<1, 128>(L, q, s);
+        e = T <= kDecWideStageTokens || T >= kDecWideStageFrom ? launch_decode<2>(L, q, s) : launch_decode<1>(L, q, s);
         if (e != cudaSuccess) return e;
         if (ev) {                           // gate/up and down share one launch: the down stage reads 0
             ace::record_stage(ev[1], s);
