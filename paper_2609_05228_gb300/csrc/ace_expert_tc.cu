@@ -268,10 +268,11 @@ __device__ __forceinline__ float wide_row_ghat(const TcParams& p, const Tile& t,
 
 // ---------------------------------------------------------------- tile hand-out
 //
-// The grouped GEMMs are persistent: a CTA's producer thread draws tile indices
-// from a counter in global memory (zeroed by the routing), so CTAs that drew
-// light tiles draw more, and hands each index to the CTA's other roles through
-// a ring in shared memory (-1 = no more tiles).
+// The grouped GEMMs are persistent: a CTA's producer thread takes its block's
+// index as the first tile and draws the next ones, from the grid size on, from a
+// counter in global memory (zeroed by the routing), so CTAs that drew light tiles
+// draw more, and hands each index to the CTA's other roles through a ring in
+// shared memory (-1 = no more tiles).
 constexpr int kTileRing = 8;
 
 struct TileRing {
@@ -439,8 +440,10 @@ __global__ void __launch_bounds__(TcCfg<EPI, STAGES, WT>::THREADS, 1) k_expert_t
             const uint64_t once_policy = l2_policy_evict_first(), reuse_policy = l2_policy_evict_normal();
             while (true) {
                 if (C::DRAW) {
-                    // drawn once the previous tile's stages are out: its latency hides behind them
-                    tile = atomicAdd(p.tile_next, 1);
+                    // the first tile is the CTA's own (a draw would delay its first load); the others are
+                    // drawn once the previous tile's stages are out: their latency hides behind them
+                    const int grid = (int)gridDim.x;
+                    tile = tile < 0 ? (int)blockIdx.x : n_tiles > grid ? grid + atomicAdd(p.tile_next, 1) : n_tiles;
                     if (tile >= n_tiles) tile = -1;
                     if (!ring_put(ring, rc, tile)) { ok = false; break; }
                 } else {
