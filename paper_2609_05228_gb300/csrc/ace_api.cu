@@ -536,7 +536,7 @@ ace_status forward_impl(ace_layer* L, const void* x, void* out, int T, ace_skip_
         ACE_CUDA(ace::launch_experts_tc(L, x, out, T, ctl, s, ev ? ev + 4 : nullptr, next), "expert launch");
     } else {
         if (ev) ACE_CUDA(ace::record_stage(ev[4], s), "event record");   // no gather stage
-        ACE_CUDA(ace::launch_experts_gemv(L, x, out, T, s, ev ? ev + 4 : nullptr), "expert launch");
+        ACE_CUDA(ace::launch_experts_gemv(L, x, out, T, ctl, s, ev ? ev + 4 : nullptr), "expert launch");
     }
     L->n_stages = ev ? ace::kNumStages : 0;
     L->last_launches = (small ? 1 : (h_ready ? 1 : 2) + ace::route_launch_count(L, T, ctl)) +

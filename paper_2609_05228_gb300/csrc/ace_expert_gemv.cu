@@ -10,8 +10,8 @@
 // latency: the chain of dependent loads, the launches (PDL) and the sums over
 // the warp (warp_sum_all). 64 tokens on the (256, 16 experts, top-4, 128) fp32
 // layer: 42 us a call with 8-token chunks, one warp_sum per token and row and
-// plain launches; 37.8 with 16-token chunks (an expert's tokens in one pass
-// where they fit) and dependent launches; 26.1 with the joint sums.
+// plain launches; 37.8 with 16-token chunks (run() says where) and dependent
+// launches; 26.1 with the joint sums.
 //   gate/up: act[r, j] = SiLU(h_t . W_gate[e, j]) * (h_t . W_up[e, j])
 //   down:    y[r, c]   = g_hat(r) * (act[r] . W_down[e, c])
 //   combine: out[t, c] = sum over t's kept slots, in rank order, of y[r, c]
@@ -278,9 +278,18 @@ __global__ void __launch_bounds__(256) k_combine(const float* __restrict__ yslot
     o[3] = from_f32<T>(acc.w);
 }
 
-// Tokens per weight pass: 16 while two blocks' staged rows of either kernel fit an SM, else 8.
+// Tokens per weight pass: 8, or 16 where experts hold more than 8 tokens, so that a second pass over
+// the weights is saved, and two blocks' staged rows of either kernel fit an SM. 16 tokens halve the
+// loads a lane has in flight and double the sums, so a layer whose experts hold few tokens loses by
+// them (fp32 calls with 8 and 16: 1600 x 1600, 16 experts, 0.5 slots an expert 73.2 and 92.2 us, 4 slots
+// 140.5 and 177.4; 1024 x 512, 64 experts, 1 slot 80.8 and 99.8). The line lies at 6 expected slots:
+// the fullest experts, which the call waits for, then hold more than 8 (1024 x 512, 16 experts, 6 slots
+// 66.0 and 60.8, 8 slots 77.7 and 69.0; 960 x 960 bf16, 64 experts, 6 slots 287 and 262). At 3 to 5 either is
+// ahead, 16 by up to 10% and 8 by up to 23% of the time.
+constexpr double kWideChunkSlots = 6.0;
+
 template <typename T>
-bool wide_chunk(const ace_layer_desc& D) {
+bool wide_chunk_fits(const ace_layer_desc& D) {
     constexpr size_t kMost = 100 << 10;
     return 16 * (size_t)D.hidden * sizeof(T) <= kMost && 16 * (size_t)D.ffn * sizeof(float) <= kMost;
 }
@@ -313,17 +322,19 @@ cudaError_t run_chunk(const ace_layer* L, const void* x, void* out, int T_, cuda
 }
 
 template <typename T>
-cudaError_t run(const ace_layer* L, const void* x, void* out, int T_, cudaStream_t s, cudaEvent_t* ev) {
-    return wide_chunk<T>(L->desc) ? run_chunk<T, 16>(L, x, out, T_, s, ev) : run_chunk<T, 8>(L, x, out, T_, s, ev);
+cudaError_t run(const ace_layer* L, const void* x, void* out, int T_, ace_skip_ctl ctl, cudaStream_t s,
+                cudaEvent_t* ev) {
+    const bool wide = wide_chunk_fits<T>(L->desc) && expected_expert_slots(L->desc, T_, ctl) >= kWideChunkSlots;
+    return wide ? run_chunk<T, 16>(L, x, out, T_, s, ev) : run_chunk<T, 8>(L, x, out, T_, s, ev);
 }
 
 template <typename T>
 cudaError_t init(const ace_layer_desc& D) {
     const int d = D.hidden, m = D.ffn;
     cudaError_t e;
-    if (wide_chunk<T>(D)) {
-        e = raise_smem_limit(k_gemv_gateup<T, 16>, (int)(16 * d * sizeof(T)));
-        return e != cudaSuccess ? e : raise_smem_limit(k_gemv_down<T, 16>, (int)(16 * m * sizeof(float)));
+    if (wide_chunk_fits<T>(D)) {
+        if ((e = raise_smem_limit(k_gemv_gateup<T, 16>, (int)(16 * d * sizeof(T)))) != cudaSuccess) return e;
+        if ((e = raise_smem_limit(k_gemv_down<T, 16>, (int)(16 * m * sizeof(float)))) != cudaSuccess) return e;
     }
     e = raise_smem_limit(k_gemv_gateup<T, 8>, (int)(8 * d * sizeof(T)));
     return e != cudaSuccess ? e : raise_smem_limit(k_gemv_down<T, 8>, (int)(8 * m * sizeof(float)));
@@ -335,9 +346,10 @@ cudaError_t gemv_init(const ace_layer* L) {
     return L->desc.dtype == ACE_BF16 ? init<__nv_bfloat16>(L->desc) : init<float>(L->desc);
 }
 
-cudaError_t launch_experts_gemv(const ace_layer* L, const void* x, void* out, int T, cudaStream_t s, cudaEvent_t* ev) {
-    if (L->desc.dtype == ACE_BF16) return run<__nv_bfloat16>(L, x, out, T, s, ev);
-    return run<float>(L, x, out, T, s, ev);
+cudaError_t launch_experts_gemv(const ace_layer* L, const void* x, void* out, int T, ace_skip_ctl ctl, cudaStream_t s,
+                                cudaEvent_t* ev) {
+    if (L->desc.dtype == ACE_BF16) return run<__nv_bfloat16>(L, x, out, T, ctl, s, ev);
+    return run<float>(L, x, out, T, ctl, s, ev);
 }
 
 }  // namespace ace

@@ -249,10 +249,19 @@ inline cudaError_t prefer_shared(K kernel) {
                                 (int)cudaSharedmemCarveoutMaxShared);
 }
 
+// Slots that an expert keeps on average, as far as the host knows: the requested
+// share of the routed slots (a token's top-1 at least), half of them in threshold
+// mode, where the kept share is not known before the call.
+inline double expected_expert_slots(const ace_layer_desc& D, int T, ace_skip_ctl ctl) {
+    const double keep = D.top_k * (ctl.mode == ACE_SKIP_RATIO ? 1.0 - (double)ctl.value : 0.5);
+    return T * (keep > 1.0 ? keep : 1.0) / D.n_experts;
+}
+
 // ---- launchers (ace_expert_gemv.cu) ----
 // ev (nullable): events recorded before gate/up, before down, before combine, after combine.
 cudaError_t gemv_init(const ace_layer* L);
-cudaError_t launch_experts_gemv(const ace_layer* L, const void* x, void* out, int T, cudaStream_t s, cudaEvent_t* ev);
+cudaError_t launch_experts_gemv(const ace_layer* L, const void* x, void* out, int T, ace_skip_ctl ctl, cudaStream_t s,
+                                cudaEvent_t* ev);
 
 constexpr int kNumStages = 7;
 

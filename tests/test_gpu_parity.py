@@ -246,6 +246,14 @@ def _layer(kind):
             spec, seed = synth.LayerSpec(256, 1024, 16, 128, dtype="bf16"), 11
         elif kind == "narrow_ffn":
             spec, seed = synth.LayerSpec(768, 16, 4, 384, dtype="bf16"), 17
+        # the CUDA-core experts: bf16 sizes that are not tensor-core tiles; rows longer than a lane's
+        # loads in flight, with 8 tokens a weight pass whatever the batch; several rows per warp
+        elif kind == "core_bf16":
+            spec, seed = synth.LayerSpec(320, 16, 4, 192, dtype="bf16"), 19
+        elif kind == "core_f32_2048":
+            spec, seed = synth.LayerSpec(2048, 8, 2, 640, dtype="f32"), 23
+        elif kind == "core_f32_1024":
+            spec, seed = synth.LayerSpec(1024, 32, 4, 512, dtype="f32"), 29
         elif kind == "few":
             # three experts of very different load, top-1: token tiles of every fill
             spec, seed = synth.LayerSpec(256, 3, 1, 128, dtype="bf16", zipf=True, zipf_beta=0.8), 13
@@ -328,6 +336,13 @@ FORWARD_CASES = [
     ("few", 769, "threshold", 0.0), ("few", 1100, "threshold", 0.0), ("few", 2051, "threshold", 0.0),
     # the combine by a block per token (hidden 512 and up; "few" and "wide" stay on the other one)
     ("narrow_ffn", 300, "ratio", 0.5), ("narrow_ffn", 97, "ratio", 0.25),   # 97: two K blocks a stage again
+    # CUDA-core experts: 8 tokens a weight pass below 6 expected slots an expert, 16 from there on
+    # (core_f32_1024: 95 and 96 tokens), experts of one pass and of several
+    ("core_bf16", 1, "ratio", 0.5), ("core_bf16", 40, "ratio", 0.5), ("core_bf16", 100, "ratio", 0.5),
+    ("core_bf16", 300, "ratio", 0.25), ("core_bf16", 64, "threshold", 0.2),
+    ("core_f32_2048", 1, "ratio", 0.0), ("core_f32_2048", 60, "ratio", 0.25), ("core_f32_2048", 300, "ratio", 0.5),
+    ("core_f32_1024", 1, "ratio", 0.5), ("core_f32_1024", 95, "ratio", 0.5), ("core_f32_1024", 96, "ratio", 0.5),
+    ("core_f32_1024", 300, "ratio", 0.25),
 ]
 
 
