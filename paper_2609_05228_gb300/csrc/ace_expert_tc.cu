@@ -684,8 +684,8 @@ struct DecParams {
 // about 0.25 us on one SM), so a lone SM streams about twice as fast with 36 KB
 // stages as with 18 KB ones: batches that retain few experts, where few SMs
 // have work, take KBS = 2 (the two K blocks of a tile are adjacent in the tiled
-// layout: one bulk copy of 32 KB), as do the largest decode batches
-// (kDecWideStageFrom); the others keep KBS = 1 (8 stages), which every SM
+// layout: one bulk copy of 32 KB), as do batches whose experts hold several
+// token tiles; the others keep KBS = 1 (8 stages), which every SM
 // streams at its share of the HBM bandwidth. 64-row tiles (M = 64 MMAs, four 8 KB
 // copies a stage) for few expected slots, which put twice as many SMs to work, were
 // taken back: 1 token 25.8 and 25.7 us a call, 4 tokens 39.8 and 40.7, 8 tokens 56.0 and
@@ -706,13 +706,21 @@ struct DecCfg {
 };
 constexpr int kDecRing = 8;             // tile indices in flight from the producer to the other roles
 constexpr int kDecRingTakers = 1 + 4 + 4;   // the MMA thread, the epilogue and the gather warps
-// Decode batches that take 2 K blocks per stage: up to 16 tokens (few distinct retained experts, few
-// SMs with work), and above 96, where popular experts hold several 16-token tiles whose weights come
-// from L2 at the stages' pace (d = 2048, Zipf routing, 256 tokens: 182.0 us a call with one K block,
-// 178.3 with two; large layer, 128 tokens: 757.0 and 750.9). Between, two are no better (24 tokens
-// 104.3 and 104.7, 64 tokens 163.1 and 163.6).
+// Decode batches that take 2 K blocks per stage (figures: us a call with one block and with two):
+// - up to 16 tokens: few distinct retained experts, few SMs with work;
+// - from 12 expected slots an expert on: experts hold several 16-token tiles, whose weights come from L2
+//   at the stages' pace (2048 x 768, 128 experts, equal shares: 12 slots 204.5 and 206.3, 16 slots 221.1 and
+//   220.0; Zipf shares: 204.5 and 197.3, 238.3 and 228.1; 8 experts of 2048 x 2048, 24 slots 57.9 and 54.7);
+// - from 97 tokens on, experts of 2^21 and more weights a matrix: HBM bounds their long loops either way
+//   where shares are equal, and popular experts hold several tiles where they are not (4096 x 2048, 256
+//   experts, 256 tokens, equal shares 1775 and 1777, Zipf shares 1509 and 1460; 2048 x 2048, 128 experts, 97
+//   tokens 423.4 and 423.7, 378.2 and 373.0; at 48 tokens 3072 x 1024, 32 experts, loses, 102.7 and 103.5).
+// The others lose by two where shares are equal (2048 x 768, 128 experts, 8 slots 188.5 and 192.6; 4096 x
+// 256, 97 tokens 161.6 and 163.6); where they are not, up to 2% either way.
 constexpr int kDecWideStageTokens = 16;
+constexpr double kDecWideStageSlots = 12.0;
 constexpr int kDecWideStageFrom = 97;
+constexpr long long kDecWideStageExpert = 1LL << 21;
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
     int v;
@@ -1688,7 +1696,9 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
         q.k = k;
         q.ready_spin = L->dbg_ready_spin > 0 ? L->dbg_ready_spin : kSpinCycles;
         q.ready_extra = L->dbg_ready_spin > 0 ? (1 << 30) : 0;
-        e = T <= kDecWideStageTokens || T >= kDecWideStageFrom ? launch_decode<2>(L, q, s) : launch_decode<1>(L, q, s);
+        const bool wide = T <= kDecWideStageTokens || expected_expert_slots(D, T, ctl) >= kDecWideStageSlots ||
+                          (T >= kDecWideStageFrom && (long long)d * m >= kDecWideStageExpert);
+        e = wide ? launch_decode<2>(L, q, s) : launch_decode<1>(L, q, s);
         if (e != cudaSuccess) return e;
         if (ev) {                           // gate/up and down share one launch: the down stage reads 0
             ace::record_stage(ev[1], s);

@@ -335,7 +335,9 @@ FORWARD_CASES = [
     ("few", 300, "threshold", 0.0), ("few", 767, "threshold", 0.0), ("few", 768, "threshold", 0.0),
     ("few", 769, "threshold", 0.0), ("few", 1100, "threshold", 0.0), ("few", 2051, "threshold", 0.0),
     # the combine by a block per token (hidden 512 and up; "few" and "wide" stay on the other one)
-    ("narrow_ffn", 300, "ratio", 0.5), ("narrow_ffn", 97, "ratio", 0.25),   # 97: two K blocks a stage again
+    ("narrow_ffn", 300, "ratio", 0.5), ("narrow_ffn", 97, "ratio", 0.25),
+    # two K blocks a decode stage from 12 expected slots an expert on ("narrow_ffn": 64 tokens; the 97 above)
+    ("narrow_ffn", 63, "ratio", 0.25), ("narrow_ffn", 64, "ratio", 0.25), ("qwen_zipf", 256, "ratio", 0.0),
     # CUDA-core experts: 8 tokens a weight pass below 6 expected slots an expert, 16 from there on
     # (core_f32_1024: 95 and 96 tokens), experts of one pass and of several
     ("core_bf16", 1, "ratio", 0.5), ("core_bf16", 40, "ratio", 0.5), ("core_bf16", 100, "ratio", 0.5),
