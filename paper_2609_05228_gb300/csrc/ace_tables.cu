@@ -292,18 +292,9 @@ __global__ void __launch_bounds__(256) k_rcr_proto(const __nv_bfloat16* __restri
 // act_e[j] = SiLU(x_e . W_gate[e, j]) * (x_e . W_up[e, j]); grid (m / 64, N),
 // each warp 8 rows j, the input row and gamma^2 in shared memory. The rows
 // pass here anyway, so the block also sums its share of ||Gamma W_gate||_F^2
-// and ||Gamma W_up||_F^2: gamma_i^2 w^2 over 8 elements in fp32, a lane's sums
-// of those as an unevaluated pair of floats (TwoSum, Knuth; about 46 bits: the
-// fp64 adds would take longer than the loads), a row's pair, the lanes and the
-// warps in fp64 in a fixed order; one partial per block and path in
-// norms[path][e][block].
-__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float q) {
-    const float s = __fadd_rn(hi, q);
-    const float b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(q, b)));
-    hi = s;
-}
-
+// and ||Gamma W_up||_F^2: gamma_i^2 w^2 over 8 elements in fp32, their sums in
+// fp64 in a fixed order (a float pair would overflow where fp64 does not); one
+// partial per block and path in norms[path][e][block].
 __global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x, const float* __restrict__ gamma2,
                                                     const __nv_bfloat16* __restrict__ w_gate,
                                                     const __nv_bfloat16* __restrict__ w_up, int d, int m,
@@ -324,7 +315,7 @@ __global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x,
         const int j = blockIdx.x * 64 + warp * 8 + t;
         const uint4* g = reinterpret_cast<const uint4*>(w_gate + (e * m + j) * (long long)d);
         const uint4* u = reinterpret_cast<const uint4*>(w_up + (e * m + j) * (long long)d);
-        float sg = 0.f, su = 0.f, gh = 0.f, gl = 0.f, uh = 0.f, ul = 0.f;
+        float sg = 0.f, su = 0.f;
 #pragma unroll 4
         for (int q = lane; q < cv; q += 32) {
             float fg[8], fu[8];
@@ -338,11 +329,9 @@ __global__ void __launch_bounds__(256) k_rcr_gateup(const float* __restrict__ x,
                 qg = fmaf(gs[q * 8 + k] * fg[k], fg[k], qg);
                 qu = fmaf(gs[q * 8 + k] * fu[k], fu[k], qu);
             }
-            two_sum_add(gh, gl, qg);
-            two_sum_add(uh, ul, qu);
+            ng += (double)qg;
+            nu += (double)qu;
         }
-        ng += (double)gh + (double)gl;
-        nu += (double)uh + (double)ul;
         sg = warp_sum(sg);
         su = warp_sum(su);
         if (lane == 0) act[e * m + j] = sg / (1.0f + expf(-sg)) * su;

@@ -66,6 +66,23 @@ def test_tables_device_chunking_and_repeatability():
     assert again[0].tobytes() == ref[0].tobytes() and again[1].tobytes() == ref[1].tobytes()
 
 
+def test_tables_device_large_weights():
+    """Norms beyond fp32's range: gate weights near 2^62, whose squares fill fp32 in sums of 8 and
+    overflow it in a row's sum (the down weights are small, so every other product stays in range).
+    The norms' sums are fp64, so the tables are as close to the oracle as for ordinary weights."""
+    w = _hetero_layer(3, d=768, n=6, m=64)
+    g = np.random.Generator(np.random.PCG64(11))
+    b = synth.bf16_bits
+    scale = 2.0 ** (-(np.arange(6) % 3))[:, None, None]
+    w.w_gate = b(np.where(g.random((6, 64, 768)) < 0.5, -1, 1) * g.uniform(0.8, 1.0, (6, 64, 768)) * scale * 2.0 ** 62)
+    w.w_up = b(g.standard_normal((6, 64, 768)) * 2.0 ** 20)
+    w.w_down = b(g.standard_normal((6, 768, 64)) * 2.0 ** -42)
+    w.gamma = b(g.uniform(0.9, 1.0, 768))
+    a, r = offline.tables_device(w, 1e-6)
+    np.testing.assert_allclose(a, O.gsp_table(w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6), rtol=2e-5)
+    np.testing.assert_allclose(r, O.rcr_table(w.router_w, w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6), rtol=2e-5)
+
+
 def test_tables_device_match_host_library_full_size():
     """The d=2048, N=128, m=768 layer of the decode and prefill benchmarks:
     GPU tables against the host library's fp64 Gram route."""
