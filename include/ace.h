@@ -355,7 +355,7 @@ ace_status ace_route_decide_noalloc(const float* logits, int T, int n_experts, i
  *   eps            the paper's epsilon (>= 0)
  *   tile_budget    not used: the weights are read in place
  *   gsp_out, rcr_out [N] host float32, written on success
- * Allocates its device scratch (O(N d + N (d / 128)^2) bytes) for the call
+ * Allocates its device scratch (O(N (d + m) + N (d / 128)^2) bytes) for the call
  * and frees it before returning; part of the work runs on a stream of its own,
  * ordered within `stream`; synchronises `stream`. Sums are taken in a fixed
  * order, so the result is the same bits on every run.

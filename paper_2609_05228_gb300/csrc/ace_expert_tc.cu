@@ -43,8 +43,6 @@ constexpr int kThreads = 192;
 struct TcParams {
     CUtensorMap tm_tok;                 // token rows [rows, K] bf16
     CUtensorMap tm_w;                   // weight rows [N * w_rows, K] bf16
-    const int32_t* offsets;             // [N+1]
-    const int32_t* dlist;               // [N]
     const int4* tt_tab;                 // token tiles (expert, first row, rows, only tile of its expert)
     const int32_t* meta;
     void* out;                          // act bf16 [rows, m], y [rows, d] (bf16) or logits
@@ -686,11 +684,12 @@ struct DecParams {
 // have work, take KBS = 2 (the two K blocks of a tile are adjacent in the tiled
 // layout: one bulk copy of 32 KB), as do batches whose experts hold several
 // token tiles; the others keep KBS = 1 (8 stages), which every SM
-// streams at its share of the HBM bandwidth. 64-row tiles (M = 64 MMAs, four 8 KB
-// copies a stage) for few expected slots, which put twice as many SMs to work, were
-// taken back: 1 token 25.8 and 25.7 us a call, 4 tokens 39.8 and 40.7, 8 tokens 56.0 and
-// 55.1; over 13 shapes at 1 to 16 tokens between 8% faster (2560 x 2048, 8 experts) and
-// 14% slower (1024 x 512, 128 experts), with no rule on the sizes that separated the two.
+// streams at its share of the HBM bandwidth. Tiles of 64 rows (M = 64 MMAs, four 8 KB
+// copies a stage) for few expected slots put twice as many SMs to work, but (us a call
+// with 128 and with 64 rows, 2048 x 768) 1 token takes 25.8 and 25.7, 4 tokens 39.8 and
+// 40.7, 8 tokens 56.0 and 55.1; over 13 shapes at 1 to 16 tokens they lie between 8%
+// faster (2560 x 2048, 8 experts) and 14% slower (1024 x 512, 128 experts), and no rule
+// on the sizes separates the two.
 template <int KBS>
 struct DecCfg {
     // warps 0-5 as in k_expert_tc; warps 6-9 gather the gate/up tiles' token
@@ -1719,8 +1718,6 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
     p1.tm_tok = L->tcm.h_gather;
     p1.w_tiles_hbm = static_cast<const uint8_t*>(L->w_gu);
     p1.w_kb = d / kBK;
-    p1.offsets = W.offsets;
-    p1.dlist = W.dlist;
     p1.tt_tab = W.tt_tab;
     p1.meta = W.meta;
     p1.perm = W.perm;

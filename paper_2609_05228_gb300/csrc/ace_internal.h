@@ -69,7 +69,8 @@ struct Workspace {
     void* y_rows = nullptr;      // [Tmax*k, d] bf16: GEMM 2's output rows of batches over 256 tokens
     void* act_bf16 = nullptr;    // [Tmax*k, m] bf16 (tensor path)
     int32_t* dec_done = nullptr; // [tiles of tt_tab] gate/up warps finished per token tile (decode kernel)
-    int4* tt_tab = nullptr;      // [N + Tmax*k/16 + 1] token tiles: (expert, first row, rows, 0)
+    int4* tt_tab = nullptr;      // [N + Tmax*k/16 + 1] token tiles: (expert, first row, rows, flag);
+                                 // flag: its expert's only tile (one-CTA prefill tables; else 0)
     int32_t* tile_cnt = nullptr; // [Tmax/8 + 1] per-token-tile tickets of the fused small-T kernel
     int32_t* sel_hist = nullptr; // [4096 + 1024] digit histograms of the threshold keys (kept zero between calls)
     uint32_t* sel_cand = nullptr;// [Tmax*k] keys of the chosen first digit (large-T threshold select)

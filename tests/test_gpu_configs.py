@@ -124,8 +124,7 @@ def test_large_layer(T, q):
 
 
 def test_large_layer_tables_device():
-    """GPU tables of the large layer (256 experts in nine chunks of the tile
-    budget, the last one ragged): A^GSP ratios of sampled experts against the
+    """GPU tables of the large layer (256 experts): A^GSP ratios of sampled experts against the
     oracle's direct fp64 products on those experts (the normalisation is one
     constant, so A[e] / A[e'] = a~_e / a~_e'), and the whole A^RCR table."""
     w, _ = _large()

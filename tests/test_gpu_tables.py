@@ -53,17 +53,23 @@ def test_tables_device_match_oracle(seed):
         np.testing.assert_allclose(r, r_ref, rtol=2e-5)
 
 
-def test_tables_device_chunking_and_repeatability():
-    """Experts processed in chunks (ragged last chunk, one expert at a time)
-    give the same bits as one chunk, and repeated calls give the same bits."""
+@pytest.mark.parametrize("d,m", [(256, 64), (256, 192), (768, 320), (512, 448)])
+def test_tables_device_sizes(d, m):
+    """Widths that are any multiple of 256 and 64: one, an odd number of and several 64-wide K blocks,
+    one and three 256-column tiles, with a number of tiles that the SMs do not share evenly."""
+    w = _hetero_layer(7, d=d, n=11, m=m)
+    a, r = offline.tables_device(w, 1e-6)
+    np.testing.assert_allclose(a, O.gsp_table(w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6), rtol=2e-5)
+    np.testing.assert_allclose(r, O.rcr_table(w.router_w, w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6), rtol=2e-5)
+
+
+def test_tables_device_repeatability():
+    """Repeated calls give the same bits, whatever the (unused) tile budget."""
     w = _hetero_layer(5, d=256, n=16, m=192)
-    per_expert = 3 * 256 * 192 * 2
     ref = offline.tables_device(w)
-    for budget in (per_expert * 3, per_expert * 5 + 7, 1):
+    for budget in (0, 0, 1, 1 << 20):
         out = offline.tables_device(w, tile_budget=budget)
         assert out[0].tobytes() == ref[0].tobytes() and out[1].tobytes() == ref[1].tobytes(), budget
-    again = offline.tables_device(w)
-    assert again[0].tobytes() == ref[0].tobytes() and again[1].tobytes() == ref[1].tobytes()
 
 
 def test_tables_device_large_weights():
@@ -80,7 +86,9 @@ def test_tables_device_large_weights():
     w.gamma = b(g.uniform(0.9, 1.0, 768))
     a, r = offline.tables_device(w, 1e-6)
     np.testing.assert_allclose(a, O.gsp_table(w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6), rtol=2e-5)
-    np.testing.assert_allclose(r, O.rcr_table(w.router_w, w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6), rtol=2e-5)
+    with np.errstate(over="ignore"):                # SiLU's exp(-u) at u near -2^67: u / inf = -0
+        r_ref = O.rcr_table(w.router_w, w.gamma, w.w_gate, w.w_up, w.w_down, 1e-6)
+    np.testing.assert_allclose(r, r_ref, rtol=2e-5)
 
 
 def test_tables_device_match_host_library_full_size():
