@@ -668,8 +668,11 @@ __device__ void fill_tile_table(const ScanOut& so, int tok_tile, int4* tt_tab, i
 constexpr int kTopkWarps = 32;
 constexpr int kHistBins = 4096;
 
+// Up to 128 experts two blocks share an SM (32 registers a thread): with one, batches of more blocks
+// than SMs took a second wave (16384 tokens 128.7 us a call with one block an SM, 125.5 with two, hidden
+// 256; 2048 wide 660.8 and 658.1).
 template <int NPL>
-__global__ void __launch_bounds__(kTopkWarps * 32) k_topk_score(float* __restrict__ logits, int n_tokens,
+__global__ void __launch_bounds__(kTopkWarps * 32, NPL <= 4 ? 2 : 1) k_topk_score(float* __restrict__ logits, int n_tokens,
                                                                 int n_exp, int k, const float* __restrict__ a_gsp,
                                                                 const float* __restrict__ a_rcr, float eps,
                                                                 int m_min, int mode, float tau,
@@ -705,8 +708,9 @@ __global__ void __launch_bounds__(kTopkWarps * 32) k_topk_score(float* __restric
                                                              // z = (sum of the slices in order + b) / temp
         if constexpr (NPL <= 8) {
             // The lane's logits stay in registers up to the top-k. The kernel is a chain of
-            // L2 round trips, so several slices are loaded before they are added.
-            constexpr int G = NPL <= 4 ? 4 : 2;
+            // L2 round trips, so two slices are loaded before they are added (four cost the
+            // registers of a second block on the SM and gained nothing).
+            constexpr int G = 2;
             float z[NPL];
             if (n_split > 1) {
                 for (int sp = 0; sp < n_split; sp += G) {
