@@ -190,16 +190,13 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
     return true;
 }
 
-// The same for a converged warp: lane 0 waits and every lane gets the result.
-// The shuffle that hands it out orders no memory accesses; the __syncwarp
-// puts the accesses of all lanes behind the phase that lane 0 observed.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, volatile int* abort_flag,
-                                               int lane) {
-    int ok = 1;
-    if (lane == 0) ok = mbar_wait_or_abort(bar, parity, err, abort_flag);
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    __syncwarp();
-    return ok != 0;
+// The same for a converged warp: every lane observes the phase itself, which
+// orders its own later accesses behind it, and all lanes get the same answer.
+// (A wait by lane 0 and a shuffle orders nothing for the other lanes, and with
+// the __syncwarp that would, it is slower: 1 token 24.5 and 23.6 us a call, 4096
+// tokens 296.4 and 291.3, large prefill 2540 and 2510.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait_or_abort(bar, parity, err, abort_flag));
 }
 
 // 1-D bulk copy global -> shared (16-byte aligned addresses, size a multiple

@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(TcCfg<EPI, STAGES, WT>::THREADS, 1) k_expert_t
                     nb[j] = in ? 16u : 0u;
                 }
                 for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, abort_flag, lane)) { ok = false; break; }
+                    if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                     const uint32_t sa = smem_u32(smem + stage * C::STAGE_BYTES) + (uint32_t)g * 128u + cx;
                     const int kx = (t.kb0 + kb) * kBK;
 #pragma unroll
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(TcCfg<EPI, STAGES, WT>::THREADS, 1) k_expert_t
             // the tile's rows and g_hat are read while its MMAs still run
             const Tile t = tile_at<C::TOKTILE, C::WTILE>(p, tile, n_base, kblocks);
             const float gh = wide_row_ghat<EPI>(p, t, quad * 32 + lane);
-            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * C::ACC_COLS);
             // lane = token row, columns = WTILE weight rows
@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
             const bool in = t.phase == 0 && r < t.nrows;
             const __nv_bfloat16* src = p.h + (size_t)(in ? p.perm[t.row0 + r] / p.k : 0) * p.d + c * 8;
             for (int kb = 0; kb < t.kblocks; kb += KBS) {
-                if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, abort_flag, lane)) { ok = false; break; }
+                if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                 if (t.phase == 0) {
                     const uint32_t sb = smem_u32(smem + stage * kDecStage + kDecA) + off;
 #pragma unroll
@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
             if (lane == 0) mbar_arrive(&ring_empty[ri]);
             if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
             if (tile < 0) break;
-            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag)) break;
             tc_fence_after();
             const DecTile t = dec_tile(p, tile, n1);
             uint32_t r[16];
@@ -1218,7 +1218,7 @@ __global__ void __launch_bounds__(PairCfg<EPI>::THREADS, 1) k_expert_pair(const 
             // the tile's rows and g_hat are read while its MMAs still run
             const Tile t = tile_at<256, 256>(p, tile, n_tiles, kblocks);
             const float gh = wide_row_ghat<EPI>(p, t, row_base + lane);
-            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256);
             epilogue_wide<EPI>(p, t, tbase, row_base, lane, gh, stg);

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_gsp_frob(const __grid_consta
         int acc = 0;
         uint32_t acc_phase = 0;
         for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag, lane)) break;
+            if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag)) break;
             tc_fence_after();
             const FrobItem it = frob_item(p, item);
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256);

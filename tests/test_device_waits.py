@@ -1,11 +1,11 @@
-"""The kernels' waits that one lane makes for its warp (a property of the
-source: the ordering they must give does not show in results that happen to
-come out right).
+"""The kernels' waits of a whole warp (a property of the source: the ordering
+they must give does not show in results that happen to come out right).
 
-Lane 0 observes an mbarrier phase and hands the answer to the other lanes by a
-shuffle, which orders no memory accesses; what the other lanes then read or
-overwrite in shared memory needs a __syncwarp behind it. mbar_wait_warp is the
-one place that does this, so no kernel may hand out such a wait by itself."""
+A lane's accesses are ordered behind an mbarrier phase that the lane has
+observed itself. Where lane 0 observes it and hands the answer out by a shuffle,
+which orders no memory accesses, the other lanes' reads and overwrites are
+ordered by nothing. mbar_wait_warp lets every lane wait, so no kernel may hand
+out such a wait by itself."""
 import re
 from pathlib import Path
 
@@ -16,10 +16,10 @@ def _without_comments(path):
     return re.sub(r"//[^\n]*|/\*.*?\*/", "", path.read_text(), flags=re.S)
 
 
-def test_helper_orders_the_other_lanes():
+def test_every_lane_waits():
     text = _without_comments(CSRC / "ace_device.cuh")
     body = re.search(r"bool mbar_wait_warp\(.*?\n}", text, re.S).group(0)
-    assert body.index("mbar_wait_or_abort(") < body.index("__shfl_sync(") < body.index("__syncwarp()")
+    assert "__all_sync(0xffffffffu, mbar_wait_or_abort(" in body and "lane" not in body
 
 
 def test_no_kernel_hands_out_a_wait_by_a_bare_shuffle():
