@@ -7,7 +7,7 @@
 //   GEMM 2 (down,    K = m): y[r, c]   = g_hat(r) * (act[r] . W_down[e, c])
 // where rows r are retained slots in expert-grouped order (the compaction's
 // permutation) and e is the slot's expert.
-//   * decode: the M operand is a tile of 128 weight rows and the N = 16
+//   * decode: the M operand is a tile of 128 (or 64) weight rows and the N = 16
 //     operand is up to 16 token rows of one expert, so each weight tile is
 //     streamed once and the MMA does the reduction the GEMV would do on the
 //     CUDA cores;
@@ -677,45 +677,44 @@ struct DecParams {
     int ready_extra;                    // added to that wait's target: 0, or unreachable (a test of the bound)
 };
 
-// A stage holds KBS K blocks of a 128-row weight tile, followed by KBS token
+// A stage holds KBS K blocks of a ROWS-row weight tile, followed by KBS token
 // boxes. Each stage costs a fixed producer / MMA / barrier round trip (measured
 // about 0.25 us on one SM), so a lone SM streams about twice as fast with 36 KB
 // stages as with 18 KB ones: batches that retain few experts, where few SMs
 // have work, take KBS = 2 (the two K blocks of a tile are adjacent in the tiled
 // layout: one bulk copy of 32 KB), as do batches whose experts hold several
 // token tiles; the others keep KBS = 1 (8 stages), which every SM
-// streams at its share of the HBM bandwidth. Tiles of 64 rows (M = 64 MMAs, four 8 KB
-// copies a stage) for few expected slots put twice as many SMs to work, but (us a call
-// with 128 and with 64 rows, 2048 x 768) 1 token takes 25.8 and 25.7, 4 tokens 39.8 and
-// 40.7, 8 tokens 56.0 and 55.1; over 13 shapes at 1 to 16 tokens they lie between 8%
-// faster (2560 x 2048, 8 experts) and 14% slower (1024 x 512, 128 experts), and no rule
-// on the sizes separates the two.
-template <int KBS>
+// streams at its share of the HBM bandwidth. The smallest, whose
+// 128-row tiles would leave SMs without work, halve the tiles: ROWS = 64 (M =
+// 64 MMAs), KBS = 4 copies of 8 KB a stage, so that twice as many SMs stream
+// stages of the same size.
+template <int KBS, int ROWS>
 struct DecCfg {
     // warps 0-5 as in k_expert_tc; warps 6-9 gather the gate/up tiles' token
     // rows from h with cp.async (one 16-byte chunk of each row per thread and
     // K block) and arrive on every stage's full barrier
     static constexpr int THREADS = kThreads + 32 * 4;
-    static constexpr int STAGES = KBS == 1 ? 8 : 6;
-    static constexpr int A1 = 128 * kBK * 2;                  // one K block of the weight tile
+    static constexpr int STAGES = KBS == 1 ? 8 : (KBS == 2 ? 6 : 5);
+    static constexpr int A1 = ROWS * kBK * 2;                 // one K block of the weight tile
     static constexpr int A = KBS * A1;
     static constexpr int B1 = 16 * kBK * 2;                   // one token box (16 rows x 64 bf16)
     static constexpr int STAGE = A + KBS * B1;
-    static constexpr int SMEM = STAGES * STAGE + 1024 + 512;
+    static constexpr int XCH = ROWS == 64 ? 2 * 16 * 16 * 4 : 0;   // up rows handed to the gate rows' warps
+    static constexpr int SMEM = STAGES * STAGE + 1024 + 512 + XCH;
 };
 constexpr int kDecRing = 8;             // tile indices in flight from the producer to the other roles
 constexpr int kDecRingTakers = 1 + 4 + 4;   // the MMA thread, the epilogue and the gather warps
 // Decode batches that take 2 K blocks per stage (figures: us a call with one block and with two):
 // - up to 16 tokens: few distinct retained experts, few SMs with work;
 // - from 12 expected slots an expert on: experts hold several 16-token tiles, whose weights come from L2
-//   at the stages' pace (2048 x 768, 128 experts, equal shares: 12 slots 204.5 and 206.3, 16 slots 221.1 and
-//   220.0; Zipf shares: 204.5 and 197.3, 238.3 and 228.1; 8 experts of 2048 x 2048, 24 slots 57.9 and 54.7);
+//   at the stages' pace (2048 x 768, 128 experts, equal shares: 12 slots 204.2 and 206.4, 16 slots 220.8 and
+//   219.4; Zipf shares: 203.2 and 196.9, 235.5 and 227.2; 8 experts of 2048 x 2048, 24 slots 56.7 and 55.6);
 // - from 97 tokens on, experts of 2^21 and more weights a matrix: HBM bounds their long loops either way
 //   where shares are equal, and popular experts hold several tiles where they are not (4096 x 2048, 256
-//   experts, 256 tokens, equal shares 1775 and 1777, Zipf shares 1509 and 1460; 2048 x 2048, 128 experts, 97
-//   tokens 423.4 and 423.7, 378.2 and 373.0; at 48 tokens 3072 x 1024, 32 experts, loses, 102.7 and 103.5).
-// The others lose by two where shares are equal (2048 x 768, 128 experts, 8 slots 188.5 and 192.6; 4096 x
-// 256, 97 tokens 161.6 and 163.6); where they are not, up to 2% either way.
+//   experts, 256 tokens, equal shares 1795 and 1796, Zipf shares 1510 and 1472; 2048 x 2048, 128 experts, 97
+//   tokens 427.6 and 427.7, 380.8 and 376.0; at 48 tokens 3072 x 1024, 32 experts, loses, 103.4 and 104.1).
+// The others lose by two where shares are equal (2048 x 768, 128 experts, 8 slots 187.9 and 191.8; 4096 x
+// 256, 97 tokens 160.9 and 163.2); where they are not, up to 3% either way.
 constexpr int kDecWideStageTokens = 16;
 constexpr double kDecWideStageSlots = 12.0;
 constexpr int kDecWideStageFrom = 97;
@@ -735,13 +734,21 @@ struct DecTile {
     int phase;    // 0 gate/up, 1 down
     int tt;       // token tile
     int e, row0, nrows;
-    int wt;       // weight tile (128 rows)
+    int wt;       // weight tile (ROWS rows)
     int kblocks;
 };
 
+// K blocks in the stage that starts at block kb: KBS, or what is left (K blocks are even: d is a
+// multiple of 256 and m of 128).
+template <int KBS>
+__device__ __forceinline__ int dec_stage_blocks(int kb, int kblocks) {
+    return KBS <= 2 ? KBS : min(KBS, kblocks - kb);
+}
+
+template <int ROWS>
 __device__ __forceinline__ DecTile dec_tile(const DecParams& p, int tile, int n1) {
     DecTile t;
-    const int wt1 = 2 * p.m / 128, wt2 = p.d / 128;
+    const int wt1 = 2 * p.m / ROWS, wt2 = p.d / ROWS;
     if (tile < n1) {
         t.phase = 0;
         t.tt = tile / wt1;
@@ -761,10 +768,9 @@ __device__ __forceinline__ DecTile dec_tile(const DecParams& p, int tile, int n1
     return t;
 }
 
-// K blocks come in whole stages: their count is even (d is a multiple of 256, m of 128).
-template <int KBS>
-__global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const __grid_constant__ DecParams p) {
-    using C = DecCfg<KBS>;
+template <int KBS, int ROWS>
+__global__ void __launch_bounds__(DecCfg<KBS, ROWS>::THREADS, 1) k_expert_decode(const __grid_constant__ DecParams p) {
+    using C = DecCfg<KBS, ROWS>;
     constexpr int kDecStages = C::STAGES, kDecStage = C::STAGE, kDecA = C::A;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -777,6 +783,9 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_empty + kDecRing);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* ring = abort_flag + 1;        // [kDecRing] tile indices, -1 = no more
+    // 64-row tiles: an epilogue warp pair's hand-over of up rows (8-byte aligned: kDecRing is even)
+    uint64_t* xch_full = reinterpret_cast<uint64_t*>(tmem_slot + 2 + kDecRing);
+    uint64_t* xch_empty = xch_full + 2;
     const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tm_act)) : "memory");
@@ -792,6 +801,10 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
             mbar_init(&ring_full[r], 1);
             mbar_init(&ring_empty[r], kDecRingTakers);
         }
+        for (int x = 0; x < 2; ++x) {
+            mbar_init(&xch_full[x], 1);
+            mbar_init(&xch_empty[x], 1);
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -806,8 +819,8 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
     const uint32_t tmem_base = *tmem_slot;
     pdl_wait();
     const int ntt = p.meta[kMetaTokTiles];
-    const int wt1 = 2 * p.m / 128;
-    const int n1 = ntt * wt1, n_tiles = n1 + ntt * (p.d / 128);
+    const int wt1 = 2 * p.m / ROWS;
+    const int n1 = ntt * wt1, n_tiles = n1 + ntt * (p.d / ROWS);
     const int done_target = 4 * wt1 + p.ready_extra;
 
     if (warp == 0) {
@@ -827,7 +840,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
                 mbar_arrive(&ring_full[ri]);
                 if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
                 if (tile >= n_tiles) break;
-                const DecTile t = dec_tile(p, tile, n1);
+                const DecTile t = dec_tile<ROWS>(p, tile, n1);
                 if (t.phase == 1) {
                     // the token tile's act rows: every gate/up epilogue warp has written
                     if (ld_acquire(p.done + t.tt) < done_target) {
@@ -845,17 +858,27 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
                 }
                 const uint8_t* wbase = t.phase == 0 ? p.w_gu : p.w_down;
                 const int wrows = t.phase == 0 ? 2 * p.m : p.d;
-                const uint8_t* w0 = wbase + ((size_t)t.e * (wrows / 128) + t.wt) * t.kblocks * 16384;
+                // the tile's first K block (a 64-row tile is half of a 16 KB block)
+                const uint8_t* w0 = wbase + ((size_t)t.e * (wrows / 128) + t.wt * ROWS / 128) * t.kblocks * 16384 +
+                                    t.wt % (128 / ROWS) * C::A1;
                 for (int kb = 0; kb < t.kblocks; kb += KBS) {
                     if (!mbar_wait_or_abort(&empty[stage], phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                     unsigned char* sa = smem + stage * kDecStage;
+                    const int nk = dec_stage_blocks<KBS>(kb, t.kblocks);
                     // gate/up: the gather warps copy the token rows (their own arrivals)
-                    mbar_expect_tx(&full[stage], t.phase == 0 ? kDecA : kDecStage);
-                    bulk_g2s(sa, w0 + (size_t)kb * 16384, kDecA, &full[stage]);
+                    mbar_expect_tx(&full[stage], nk * (t.phase == 0 ? C::A1 : C::A1 + C::B1));
+                    if (ROWS == 128) {
+                        bulk_g2s(sa, w0 + (size_t)kb * 16384, KBS * 16384, &full[stage]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < KBS; ++j)
+                            if (j < nk) bulk_g2s(sa + j * C::A1, w0 + (size_t)(kb + j) * 16384, C::A1, &full[stage]);
+                    }
                     if (t.phase == 1) {
 #pragma unroll
                         for (int j = 0; j < KBS; ++j)
-                            tma_load_2d(sa + kDecA + j * C::B1, &p.tm_act, &full[stage], (kb + j) * kBK, t.row0);
+                            if (j < nk)
+                                tma_load_2d(sa + kDecA + j * C::B1, &p.tm_act, &full[stage], (kb + j) * kBK, t.row0);
                     }
                     ++issued;
                     if (++stage == kDecStages) { stage = 0; phase ^= 1u; }
@@ -874,7 +897,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(128, 16);
+            constexpr uint32_t idesc = idesc_bf16(ROWS, 16);
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -888,7 +911,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
                 mbar_arrive(&ring_empty[ri]);
                 if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
                 if (tile < 0) break;
-                const DecTile t = dec_tile(p, tile, n1);
+                const DecTile t = dec_tile<ROWS>(p, tile, n1);
                 if (!mbar_wait_or_abort(&acc_empty[acc], acc_phase ^ 1u, p.err, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 16);
@@ -898,8 +921,10 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     tc_fence_after();
                     const uint32_t s_addr = smem_u32(smem + stage * kDecStage);
+                    const int nk = dec_stage_blocks<KBS>(kb, t.kblocks);
 #pragma unroll
                     for (int j = 0; j < KBS; ++j) {
+                        if (j >= nk) break;
                         const uint32_t a_addr = s_addr + j * C::A1;               // weight tile kb + j
                         const uint32_t b_addr = s_addr + kDecA + j * C::B1;       // its token box
                         const uint64_t ad = smem_desc_sw128(a_addr), bd = smem_desc_sw128(b_addr);
@@ -943,7 +968,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
             if (lane == 0) mbar_arrive(&ring_empty[ri]);
             if (++ri == kDecRing) { ri = 0; rph ^= 1u; }
             if (tile < 0) break;
-            const DecTile t = dec_tile(p, tile, n1);
+            const DecTile t = dec_tile<ROWS>(p, tile, n1);
             const bool in = t.phase == 0 && r < t.nrows;
             const __nv_bfloat16* src = p.h + (size_t)(in ? p.perm[t.row0 + r] / p.k : 0) * p.d + c * 8;
             for (int kb = 0; kb < t.kblocks; kb += KBS) {
@@ -952,7 +977,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
                     const uint32_t sb = smem_u32(smem + stage * kDecStage + kDecA) + off;
 #pragma unroll
                     for (int j = 0; j < KBS; ++j)
-                        cp_async16(sb + j * C::B1, src + (kb + j) * kBK, in ? 16u : 0u);
+                        if (kb + j < t.kblocks) cp_async16(sb + j * C::B1, src + (kb + j) * kBK, in ? 16u : 0u);
                 }
                 cp_async_arrive_noinc(&full[stage]);
                 if (++stage == kDecStages) { stage = 0; phase ^= 1u; }
@@ -967,6 +992,7 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
         uint32_t acc_phase = 0;
         int ri = 0;
         uint32_t rph = 0;
+        uint32_t xch_phase = 0;
         while (true) {
             int tile = -1, go = 1;
             if (lane == 0) {
@@ -981,11 +1007,43 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
             if (tile < 0) break;
             if (!mbar_wait_warp(&acc_full[acc], acc_phase, p.err, abort_flag)) break;
             tc_fence_after();
-            const DecTile t = dec_tile(p, tile, n1);
+            const DecTile t = dec_tile<ROWS>(p, tile, n1);
             uint32_t r[16];
             tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 16), r);
             tmem_ld_wait();
-            if (t.phase == 0) {
+            if (ROWS == 64 && t.phase == 0) {
+                // M = 64: this warp's rows sit in its first 16 lanes, gate rows of FFN block
+                // 2 * wt + quad / 2 for an even quad, its up rows for the odd one, which hands
+                // them over in shared memory
+                const int pr = quad >> 1;
+                float* xch = reinterpret_cast<float*>(smem + kDecStages * kDecStage + 512) + pr * 256;
+                if (quad & 1) {
+                    if (!mbar_wait_warp(&xch_empty[pr], xch_phase ^ 1u, p.err, abort_flag)) break;
+                    if (lane < 16) {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) xch[c * 16 + lane] = __uint_as_float(r[c]);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&xch_full[pr]);
+                } else {
+                    if (!mbar_wait_warp(&xch_full[pr], xch_phase, p.err, abort_flag)) break;
+                    if (lane < 16) {
+                        const int j = (t.wt * 2 + pr) * 16 + lane;
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            if (c < t.nrows)
+                                p.act[(size_t)(t.row0 + c) * p.m + j] =
+                                    __float2bfloat16_rn(silu(__uint_as_float(r[c])) * xch[c * 16 + lane]);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&xch_empty[pr]);
+                    fence_proxy_async_global();      // act is read by the TMA of down tiles
+                    __threadfence();
+                    __syncwarp();
+                }
+                xch_phase ^= 1u;
+                if (lane == 0) atomicAdd(p.done + t.tt, 1);
+            } else if (t.phase == 0) {
                 // rows: 16 gate then 16 up of FFN block (4 * wt + quad); SwiGLU into act
                 const int j = (t.wt * 4 + quad) * 16 + (lane & 15);
 #pragma unroll
@@ -1000,10 +1058,11 @@ __global__ void __launch_bounds__(DecCfg<KBS>::THREADS, 1) k_expert_decode(const
                 __syncwarp();
                 if (lane == 0) atomicAdd(p.done + t.tt, 1);
             } else {
-                const int col = t.wt * 128 + quad * 32 + lane;
+                // a warp's rows: 32 lanes (M = 128) or the first 16 (M = 64)
+                const int col = t.wt * ROWS + quad * (ROWS / 4) + lane;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
-                    if (c < t.nrows)
+                    if (lane < ROWS / 4 && c < t.nrows)
                         p.y[(size_t)(t.row0 + c) * p.d + col] = p.ghat[p.perm[t.row0 + c]] * __uint_as_float(r[c]);
                 }
             }
@@ -1485,17 +1544,35 @@ cudaError_t set_combine_attr(int d) {
     return e != cudaSuccess ? e : prefer_shared(k_combine_norm<KMAX, NORM>);
 }
 
-template <int KBS>
+template <int KBS, int ROWS>
 cudaError_t set_decode_attr() {
-    cudaError_t e = cudaFuncSetAttribute(k_expert_decode<KBS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         DecCfg<KBS>::SMEM);
-    return e != cudaSuccess ? e : prefer_shared(k_expert_decode<KBS>);
+    cudaError_t e = cudaFuncSetAttribute(k_expert_decode<KBS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         DecCfg<KBS, ROWS>::SMEM);
+    return e != cudaSuccess ? e : prefer_shared(k_expert_decode<KBS, ROWS>);
 }
 
-template <int KBS>
+template <int KBS, int ROWS>
 cudaError_t launch_decode(const ace_layer* L, const DecParams& q, cudaStream_t s) {
-    using C = DecCfg<KBS>;
-    return launch_pdl(k_expert_decode<KBS>, dim3(L->num_sms), dim3(C::THREADS), C::SMEM, s, q);
+    using C = DecCfg<KBS, ROWS>;
+    return launch_pdl(k_expert_decode<KBS, ROWS>, dim3(L->num_sms), dim3(C::THREADS), C::SMEM, s, q);
+}
+
+// 64-row weight tiles, by the gate/up work in rounds of 128-row tiles over the SMs (expected
+// distinct experts of the slots expected to be kept). Up to half a round, halving the tiles puts
+// twice as many SMs to work (us a call with 128 and 64 rows; 2048 x 768, 128 experts, 1 token: 25.0 and
+// 23.4; 1024 x 512, 32 experts, 4 tokens: 20.8 and 19.7; 256 x 128: the same). From there to a round the
+// halves need a second round (2 tokens: 25.2 and 25.6; 512 x 256, 32 experts, 8 tokens: 18.2 and 19.4); then,
+// with a K loop long enough to hide a tile's own cost, they fill the last round better (4 / 6 / 8
+// tokens: 39.4 and 38.2, 48.0 and 46.7, 55.7 and 54.6; large layer, 1 token: 49.8 and 48.1; 3072 x 768, 3
+// tokens: 45.4 and 43.1), until HBM bounds the kernel (12 tokens: 73.3 and 73.9). Shorter K loops do not:
+// 1024 x 512, 128 experts, 8 tokens 27.3 and 29.9; 1280 to 1792 wide between 7% faster and 6% slower.
+bool dec_half_tiles(const ace_layer* L, int T, ace_skip_ctl ctl) {
+    const ace_layer_desc& D = L->desc;
+    if (T > kDecWideStageTokens) return false;
+    const double slots = expected_expert_slots(D, T, ctl) * D.n_experts;
+    const double experts = T == 1 ? slots : D.n_experts * (1.0 - pow(1.0 - 1.0 / D.n_experts, slots));
+    const double rounds = experts * (2 * D.ffn / 128) / L->num_sms;
+    return rounds <= 0.5 || (D.hidden >= 2048 && rounds >= 0.8 && rounds <= 2.5);
 }
 
 // Experts per router tile: one 128-column tile covers up to 128 experts.
@@ -1593,8 +1670,9 @@ cudaError_t tc_init(ace_layer* L) {
     if ((e = set_attr<1, kStagesWide, 256>()) != cudaSuccess) return e;
     if ((e = set_attr<2, kStagesWide, 256>()) != cudaSuccess) return e;
     if ((e = set_attr<2, kStagesNarrow, 128>()) != cudaSuccess) return e;
-    if ((e = set_decode_attr<1>()) != cudaSuccess) return e;
-    if ((e = set_decode_attr<2>()) != cudaSuccess) return e;
+    if ((e = set_decode_attr<1, 128>()) != cudaSuccess) return e;
+    if ((e = set_decode_attr<2, 128>()) != cudaSuccess) return e;
+    if ((e = set_decode_attr<4, 64>()) != cudaSuccess) return e;
     if ((e = set_pair_attr((const void*)k_expert_pair<0>)) != cudaSuccess) return e;
     if ((e = set_pair_attr((const void*)k_expert_pair<1>)) != cudaSuccess) return e;
     int c0 = 0, c1 = 0;
@@ -1697,7 +1775,9 @@ cudaError_t launch_experts_tc(const ace_layer* L, const void* x, void* out, int 
         q.ready_extra = L->dbg_ready_spin > 0 ? (1 << 30) : 0;
         const bool wide = T <= kDecWideStageTokens || expected_expert_slots(D, T, ctl) >= kDecWideStageSlots ||
                           (T >= kDecWideStageFrom && (long long)d * m >= kDecWideStageExpert);
-        e = wide ? launch_decode<2>(L, q, s) : launch_decode<1>(L, q, s);
+        e = dec_half_tiles(L, T, ctl) ? launch_decode<4, 64>(L, q, s)
+            : wide                    ? launch_decode<2, 128>(L, q, s)
+                                      : launch_decode<1, 128>(L, q, s);
         if (e != cudaSuccess) return e;
         if (ev) {                           // gate/up and down share one launch: the down stage reads 0
             ace::record_stage(ev[1], s);

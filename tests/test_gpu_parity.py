@@ -325,10 +325,11 @@ FORWARD_CASES = [
     ("qwen_temp", 64, "ratio", 0.5), ("qwen_temp", 600, "ratio", 0.625), ("qwen_temp", 48, "threshold", 0.1),
     ("qwen", 256, "ratio", 0.5), ("qwen", 257, "ratio", 0.5),          # both sides of the small-batch path
     ("wide", 40, "ratio", 0.5), ("wide", 700, "ratio", 0.5), ("wide", 256, "threshold", 0.05),
-    # the smallest decode batches; "few" and "narrow_ffn": down projections of 2 and 6 K blocks,
-    # one and three stages of two
+    # decode with 64-row weight tiles (few expected slots) and the first sizes on 128-row ones;
+    # "few" and "narrow_ffn": down projections of 2 and 6 K blocks, half a stage left over
     ("qwen", 2, "ratio", 0.25), ("qwen", 6, "ratio", 0.5), ("qwen", 7, "ratio", 0.5),
-    ("narrow_ffn", 1, "ratio", 0.0), ("narrow_ffn", 9, "ratio", 0.5), ("few", 1, "threshold", 0.0),
+    ("qwen", 8, "threshold", 0.11), ("narrow_ffn", 1, "ratio", 0.0), ("narrow_ffn", 9, "ratio", 0.5),
+    ("few", 1, "threshold", 0.0),
     ("few", 16, "threshold", 0.0), ("few", 17, "threshold", 0.0),
     # one CTA per tile (below 256 slots an expert on average) with experts of one and of several
     # tiles; CTA pairs from 768 tokens on, with last tiles that leave gather warps without rows
